@@ -159,7 +159,7 @@ bool k2_newton_on(const mg_config *c)
 }
 
 struct Layout {
-    size_t X, SRC, R, D, PB, RT, BY, partial, scal, Z, ZR, Gpsi, GW, gj, own, child, total;
+    size_t X, SRC, R, PB, RT, BY, partial, scal, Z, ZR, Gpsi, GW, gj, own, child, total;
     int dense, mpsi, mw, has_child;
     std::vector<size_t> eA, eB, f, c;
 };
@@ -175,7 +175,6 @@ Layout layout_for(const mg_config *c)
     L.X = take(4 * N * 8);
     L.SRC = take(5 * N * 8);
     L.R = take(5 * N * 8);
-    L.D = take(4 * N * 8);
     if (c->npunct > 0) L.PB = take(N * 8);
     if (c->bc == MG_BC_ROBIN) L.RT = take((size_t)(c->n[0] + 4) * (c->n[1] + 4) * (c->n[2] + 4) * 8);
     if (has_bowen_york(c)) L.BY = take(6 * N * 8);
@@ -186,7 +185,9 @@ Layout layout_for(const mg_config *c)
         L.f.push_back(take(4 * Nl * tb));
         L.c.push_back(take(2 * Nl * tb));
     }
-    L.partial = take((size_t)kRedBlocks * 8 * 8);
+    Geo g0{};
+    for (int a = 0; a < 3; ++a) g0.n[a] = c->n[a];
+    L.partial = take(std::max((size_t)kRedBlocks * 8, (size_t)outer_ctas(g0, outer_grid(g0)) * 5) * 8);
     L.scal = take(sizeof(Scalars));
     if (k2_newton_on(c)) {
         L.Z = take(4 * N * tb);
@@ -520,7 +521,6 @@ mg_status mg_create(const mg_config *cfg, void *cuda_stream, void *workspace, si
         x->X = (double *)(b + lay.X);
         x->SRC = (double *)(b + lay.SRC);
         x->R = (double *)(b + lay.R);
-        x->D = (double *)(b + lay.D);
         x->dense = lay.dense;
         x->mpsi = lay.mpsi;
         x->mw = lay.mw;
@@ -940,8 +940,7 @@ static mg_status mg_time_kernel_impl(mg_ctx *x, int which, int reps, double *ms_
     double N = (double)x->N, s = (double)x->tbytes, b = 0.0;
     if (which == 0) b = 0.5 * 14.0 * s * N;               // half of a two-colour sweep: (2 F + 6) s per cell (algorithmic)
     else if (which == 1) b = (10.0 * s + 4.0 * s / 8.0) * N; // read e, f, a, b; write the coarse rhs
-    else if (which == 2) b = (3.0 + 4.0 + 4.0 + 4.0 + 5.0 + 5.0) * 8.0 * N; // A: W -> q/div; B: u, W, q/div, 5 sources -> 5
-    else b = (4.0 + 4.0 + 5.0 + 5.0) * 8.0 * N;                   // B: read u, W, q/div, 5 sources; write 5
+    else b = (4.0 + 5.0 + 5.0) * 8.0 * N;                         // read u, W, 5 sources; write 5
     if (ms_per_launch) *ms_per_launch = ms / reps;
     if (bytes_per_launch) *bytes_per_launch = b;
     return MG_OK;

@@ -154,50 +154,6 @@ Coef<T> make_coef(const Geo &g, int order, double omega = 1.0)
     return cf;
 }
 
-inline OuterCoef make_outer_coef(const Geo &g, int order)
-{
-    OuterCoef o;
-    const double w0 = order == 2 ? -2.0 : -30.0 / 12.0;
-    o.k0 = 0.0;
-    for (int a = 0; a < 3; ++a) {
-        const double h = g.h[a], h2 = h * h;
-        o.c1[a] = (order == 2 ? 0.5 : 8.0 / 12.0) / h;
-        o.c2[a] = order == 2 ? 0.0 : (1.0 / 12.0) / h;
-        o.k1[a] = (order == 2 ? 1.0 : 16.0 / 12.0) / h2;
-        o.nk2[a] = order == 2 ? 0.0 : -(1.0 / 12.0) / h2;
-        o.k0 += w0 / h2;
-        o.q1[a] = o.c1[a] / 3.0;
-        o.q2[a] = o.c2[a] / 3.0;
-    }
-    for (int A = 0; A < 3; ++A) {
-        for (int a = 0; a < 3; ++a) {
-            const double s = a == A ? 4.0 / 3.0 : 1.0;
-            o.m1[A][a] = s * o.k1[a];
-            o.nm2[A][a] = s * o.nk2[a];
-        }
-        o.m0[A] = o.k0 + w0 / (3.0 * g.h[A] * g.h[A]);
-    }
-    return o;
-}
-
-// Block split of the FP64 residual pass B: shell blocks first, then interior-box blocks; at most
-// kRedBlocks blocks in all (one reduction partial each).  A periodic shell cell costs about an
-// interior cell (q form, wrapped); a Robin shell cell takes the tensor-product form with boundary
-// values, several times the arithmetic, so Robin boxes give the shell up to half the blocks.
-inline Regions outer_regions(const Geo &g, int order, int robin, int *grid)
-{
-    Regions r;
-    r.G = order / 2;
-    long long ix = g.n[0] - 2 * r.G, iy = g.n[1] - 2 * r.G, iz = g.n[2] - 2 * r.G;
-    size_t nint = (ix > 0 && iy > 0 && iz > 0) ? (size_t)ix * iy * iz : 0;
-    size_t nsh = shell_count(g.n, r.G);
-    int bs = nsh ? grid_for(nsh, robin ? kRedBlocks / 2 : 152, kThreads) : 0;
-    int bi = nint ? grid_for(nint, kRedBlocks - bs, kThreads) : 0;
-    r.nblk_sh = bs;
-    *grid = std::max(1, bi + bs);
-    return r;
-}
-
 // Dense coarsest-level solve: available when the bordered W system has at most kDenseMaxW rows.
 inline bool dense_eligible(const int nc[3], int periodic)
 {
@@ -247,7 +203,6 @@ struct mg_ctx {
     double *X = nullptr;     // 4N: u, Wx, Wy, Wz
     double *SRC = nullptr;   // 5N: rho0, rho2, Sx, Sy, Sz
     double *R = nullptr;     // 5N: outer pass-1 output
-    double *D = nullptr;     // 4N: q_0, q_1, q_2, div W of the FP64 residual's pass A
     int dense = 0;           // 1: the coarsest level is solved with the dense inverses below
     int fused = 0;           // 1: the next-to-coarsest level's cycle runs in one CTA (k_coarse_cycle)
     int mpsi = 0, mw = 0;    // orders of the (bordered) psi and W systems

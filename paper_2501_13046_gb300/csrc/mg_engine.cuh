@@ -214,28 +214,23 @@ mg_status enqueue_cycle(mg_ctx *x, int l, bool zero)
 template <typename T, int ORDER, int BC>
 mg_status enqueue_vcycle(mg_ctx *x, bool first) { return enqueue_cycle<T, ORDER, BC>(x, 0, first); }
 
-// FP64 residual pass 1 (pass A: q, div W; pass B: R and the integrability sums), then the
-// final reduction of the sums.
-// Pass B finishes the outer scalars in its last block (sums, K^2, m_i).
+// What the fused FP64 residual finishes in its last block: the sums, K^2, m_i.
 inline OuterFin outer_fin(mg_ctx *x)
 {
     return OuterFin{x->scal, x->cfg.k_mode == MG_K_INTEGRABILITY, x->cfg.bc == MG_BC_PERIODIC, x->cfg.K * x->cfg.K};
 }
 
-template <int ORDER, int BC>
-mg_status enqueue_outer_pass1(mg_ctx *x)
+// FP64 residual pass 1: R and the integrability sums.  (Templated on T although the kernel is not: each
+// translation unit has its own kernel and attributes, so each needs its own launching function.)
+template <typename T, int ORDER, int BC>
+mg_status enqueue_outer_pass1(mg_ctx *x, const OuterFin &fin)
 {
-    LevelBufs &L0 = x->lev[0];
-    Coef<double> cf = make_coef<double>(L0.geo, x->cfg.order);
-    OuterCoef oc = make_outer_coef(L0.geo, x->cfg.order);
-    int gb = 0;
-    Regions rg = outer_regions(L0.geo, ORDER, x->cfg.bc == MG_BC_ROBIN, &gb);
-    with_bc<BC>([&](auto B) {
-        k_outer_div<ORDER, decltype(B)::value><<<grid_for(x->N, 1 << 24), kThreads, 0, x->stream>>>(L0.geo, oc, x->X,
-                                                                                                      x->D);
-        k_outer_pass1q<ORDER, decltype(B)::value><<<gb, kThreads, 0, x->stream>>>(L0.geo, cf, oc, x->X, x->D, x->SRC,
-                                                                                  x->R, x->partial, rg, outer_fin(x));
-    });
+    const Geo &g = x->lev[0].geo;
+    const OuterGrid tg = outer_grid(g);
+    const OuterIn in{x->X, x->X + x->N, x->SRC, x->SRC + x->N, x->SRC + 2 * x->N};
+    k_outer_residual<ORDER, BC><<<outer_ctas(g, tg), kOutThreads, outer_smem_bytes<ORDER>(), x->stream>>>(
+        g, make_coef<double>(g, x->cfg.order), make_outer_int(g, x->cfg.order), in, x->R, x->R + 4 * x->N, x->partial,
+        tg, fin);
     CK(cudaGetLastError());
     return MG_OK;
 }
@@ -245,7 +240,7 @@ template <typename T, int ORDER, int BC>
 mg_status enqueue_residual(mg_ctx *x, double *HM)
 {
     LevelBufs &L0 = x->lev[0];
-    CKS(enqueue_outer_pass1<ORDER, BC>(x));
+    CKS(enqueue_outer_pass1<T, ORDER, BC>(x, outer_fin(x)));
     int g1 = grid_for(x->N, kRedBlocks);
     k_outer_pass2<T><<<g1, kThreads, 0, x->stream>>>(L0.geo, x->X, x->R, x->SRC, x->scal, (T *)L0.f, (T *)L0.c, HM,
                                                      x->partial, L0.split, 1);
@@ -377,6 +372,9 @@ mg_status engine_prepare(mg_ctx *x)
             cudaFuncSetAttribute(k_restrict_tile<T, ORDER, BC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)tile_restrict_smem_bytes<T, ORDER>()) != cudaSuccess)
             st = fail(MG_ERR_CUDA, "cudaFuncSetAttribute(tiled kernels)");
+        if (cudaFuncSetAttribute(k_outer_residual<ORDER, BC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)outer_smem_bytes<ORDER>()) != cudaSuccess)
+            st = fail(MG_ERR_CUDA, "cudaFuncSetAttribute(k_outer_residual)");
     });
     return st;
 }
@@ -408,17 +406,8 @@ mg_status engine_time_kernel(mg_ctx *x, int which, int reps, float *ms)
             L.curB = 0;   // residual of eA
             CKS(enqueue_restrict<T, ORDER, BC>(x, 0));
             L.curB = keep;
-        } else if (which == 2) {
-            CKS(enqueue_outer_pass1<ORDER, BC>(x));
-        } else {   // pass B alone (reads pass A's q, div W from the last residual evaluation)
-            Coef<double> cd = make_coef<double>(L.geo, x->cfg.order);
-            OuterCoef oc = make_outer_coef(L.geo, x->cfg.order);
-            int gb = 0;
-            Regions rg = outer_regions(L.geo, ORDER, x->cfg.bc == MG_BC_ROBIN, &gb);
-            with_bc<BC>([&](auto B) {
-                k_outer_pass1q<ORDER, decltype(B)::value><<<gb, kThreads, 0, x->stream>>>(
-                    L.geo, cd, oc, x->X, x->D, x->SRC, x->R, x->partial, rg, OuterFin{nullptr, 0, 0, 0.0});
-            });
+        } else {   // the fused residual, with (2) or without (3) the reduction of its sums
+            CKS(enqueue_outer_pass1<T, ORDER, BC>(x, which == 2 ? outer_fin(x) : OuterFin{nullptr, 0, 0, 0.0}));
         }
     }
     CK(cudaGetLastError());

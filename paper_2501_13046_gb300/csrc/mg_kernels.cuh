@@ -958,8 +958,7 @@ __device__ __forceinline__ void block_max(double (&v)[NV], double *out)
 }
 
 // Last-block finalisation of a grid reduction: every block has stored its row of NV partials; the
-// block whose ticket comes last reduces all rows in the order and tree of k_finalize_sum /
-// k_finalize_max (blockDim.x = 256 there and here, so the result is the same) into out, and
+// block whose ticket comes last reduces all rows (in a fixed order: deterministic) into out, and
 // returns true in all its threads.  atomicInc wraps the ticket back to 0 for the next launch.
 template <int NV, bool MAX>
 __device__ __forceinline__ bool finalize_last(const double *partial, int nblocks, double *out, unsigned int *ticket)
@@ -1056,22 +1055,7 @@ static __global__ void __launch_bounds__(256) k_flag_nonfinite(const double *__r
     if (__syncthreads_or(bad) && threadIdx.x == 0) atomicOr(flag, 1u);
 }
 
-// Final single-block reduction of per-block partial sums: partial[b * NV + a].
-template <int NV>
-__global__ void k_finalize_sum(const double *__restrict__ partial, int nblocks, double *__restrict__ out)
-{
-    double v[NV];
-#pragma unroll
-    for (int a = 0; a < NV; ++a) v[a] = 0.0;
-    for (int b = threadIdx.x; b < nblocks; b += blockDim.x)
-#pragma unroll
-        for (int a = 0; a < NV; ++a) v[a] += partial[b * NV + a];
-    double r[NV];
-    block_sum<NV>(v, r);
-    if (threadIdx.x == 0)
-        for (int a = 0; a < NV; ++a) out[a] = r[a];
-}
-
+// Final single-block reduction of per-block partial maxima: partial[b * NV + a].
 template <int NV>
 __global__ void k_finalize_max(const double *__restrict__ partial, int nblocks, double *__restrict__ out)
 {
@@ -1177,11 +1161,9 @@ __global__ void __launch_bounds__(256) k_update(Geo g, double *__restrict__ x, c
 }
 
 // ---------------------------------------------------------------------------------------
-// Outer FP64 residual, pass 1.  Per cell:
-//   R0 = Lap u + (1/8) psi^-7 AtAt + 2 pi (rho0 psi^5 + rho2 psi)       (F_psi before the K^2 term)
-//   R1..3 = Lap W_i + (1/3) d_i d_j W_j - 8 pi psi^6 S_i                   (F_W before adding m_i)
-//   R4 = AtAt (the linearisation coefficient c is formed from it in pass 2)
-// and block partial sums of (1/8) psi^-7 AtAt + 2 pi (rho0 psi^5 + rho2 psi), psi^5, 8 pi psi^6 S_i.
+// Lap u, AtAt and the momentum operator (mom) at a cell, the direct FP64 form: every stencil,
+// the mixed terms as tensor products, from accessors of the 4 fields.  by: the cell's Bowen-York
+// part of At_ij (stride N) or null.
 template <int ORDER, class F>
 __device__ __forceinline__ void outer_cell(const F &u, const F &w0, const F &w1, const F &w2, const Coef<double> &cf,
                                            double &lu, double &aa, double mom[3], const double *by = nullptr,
@@ -1221,13 +1203,6 @@ __device__ __forceinline__ void outer_cell(const F &u, const F &w0, const F &w1,
     mom[0] = Je[1];
     mom[1] = Je[2];
     mom[2] = Je[3];
-}
-
-// K^2 (integrability or fixed) and the momentum-source means from the pass-1 sums.
-static __global__ void k_outer_scalars(Scalars *s, size_t N, int kmode_integrability, double K2_fixed, int periodic)
-{
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    outer_scalars(s, N, kmode_integrability, K2_fixed, periodic);
 }
 
 // Pass 2: final residuals, norm partials, inner right-hand side and coefficients in T:

@@ -15,7 +15,7 @@ namespace {
 
 constexpr size_t kNoallocMaxCells = 64 * 64 * 64;                 // 262,144 cells
 constexpr size_t kNoallocR = 4 * kNoallocMaxCells;                // pass-1 output, 4 FP64 fields
-constexpr size_t kNoallocPartials = (size_t)kRedBlocks * 8;       // block partials
+constexpr size_t kNoallocPartials = (size_t)kRedBlocks * 8;       // block partials (5 per CTA of the residual, 4 of the norms)
 constexpr size_t kNoallocScalars = 64;                            // >= sizeof(Scalars) / 8
 constexpr size_t kNoallocDoubles = kNoallocR + kNoallocPartials + kNoallocScalars;   // 8.47 MB
 static_assert(sizeof(Scalars) <= kNoallocScalars * sizeof(double), "scalar slot too small");
@@ -41,52 +41,6 @@ mg_status scratch_address(double **out)
     }
     *out = g_addr[dev];
     return MG_OK;
-}
-
-// Pass 1 of the outer residual with the state and sources in separate caller arrays.
-template <int ORDER, int BC>
-__global__ void __launch_bounds__(256) k_noalloc_pass1(Geo g, Coef<double> cf, const double *__restrict__ u,
-                                                       const double *__restrict__ W, const double *__restrict__ rho0,
-                                                       const double *__restrict__ rho2, const double *__restrict__ S,
-                                                       double *__restrict__ R, double *__restrict__ partial)
-{
-    const size_t N = (size_t)g.n[0] * g.n[1] * g.n[2];
-    const int sy = g.n[0], sz = g.n[0] * g.n[1];
-    double acc[5] = {0, 0, 0, 0, 0};
-    for (size_t p = blockIdx.x * (size_t)blockDim.x + threadIdx.x; p < N; p += (size_t)gridDim.x * blockDim.x) {
-        int i = (int)(p % g.n[0]);
-        size_t rest = p / g.n[0];
-        int j = (int)(rest % g.n[1]);
-        int k = (int)(rest / g.n[1]);
-        double lu, aa, mom[3];
-        if (is_interior(g, i, j, k, halo<ORDER>())) {
-            AccI<double> a0{u + p, sy, sz}, a1{W + p, sy, sz}, a2{W + N + p, sy, sz}, a3{W + 2 * N + p, sy, sz};
-            outer_cell<ORDER>(a0, a1, a2, a3, cf, lu, aa, mom);
-        } else {
-            AccB<double, BC> a0{u, 0, &g, i, j, k}, a1{W, 1, &g, i, j, k}, a2{W + N, 2, &g, i, j, k},
-                a3{W + 2 * N, 3, &g, i, j, k};
-            outer_cell<ORDER>(a0, a1, a2, a3, cf, lu, aa, mom);
-        }
-        double psi = psi_background(g, i, j, k) + u[p];
-        double r0 = rho0[p], r2 = rho2 ? rho2[p] : 0.0;
-        double ip = 1.0 / psi;
-        double p2 = psi * psi, p5 = p2 * p2 * psi, p6 = p5 * psi;
-        double ip2 = ip * ip, ip4 = ip2 * ip2, ip7 = ip4 * ip2 * ip;
-        double nonlin = 0.125 * aa * ip7 + 2.0 * kPi * (r0 * p5 + r2 * psi);
-        R[p] = lu + nonlin;
-        acc[0] += nonlin;
-        acc[1] += p5;
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            double s = 8.0 * kPi * p6 * S[a * N + p];
-            R[(1 + a) * N + p] = mom[a] - s;
-            acc[2 + a] += s;
-        }
-    }
-    double r[5];
-    block_sum<5>(acc, r);
-    if (threadIdx.x == 0)
-        for (int a = 0; a < 5; ++a) partial[blockIdx.x * 5 + a] = r[a];
 }
 
 // Block partial maxima of |H| and |M_i| (nothing else is written).
@@ -178,11 +132,19 @@ extern "C" mg_status mg_residual_norms_noalloc(const mg_config *cfg, const doubl
     Scalars *sc = reinterpret_cast<Scalars *>(scratch + kNoallocR + kNoallocPartials);
     // the scalars are read back below: start them at zero on every call
     CK(cudaMemsetAsync(sc, 0, sizeof(Scalars), st));
-    Coef<double> cf = make_coef<double>(g, cfg->order);
     const int g1 = grid_for(N, kRedBlocks);
+    const OuterGrid tg = outer_grid(g);
+    if ((size_t)outer_ctas(g, tg) * 5 > kNoallocPartials)   // (at most 1824 CTAs on 262144 cells)
+        return fail(MG_ERR_INVALID_ARG, "mg_residual_norms_noalloc: too many tiles for the static scratch");
+    const OuterIn in{u, W, rho0, rho2, S};
+    const OuterFin fin{sc, cfg->k_mode == MG_K_INTEGRABILITY, cfg->bc == MG_BC_PERIODIC, cfg->K * cfg->K};
+    cudaError_t attr = cudaSuccess;
     auto launch1 = [&](auto O, auto B) {
-        k_noalloc_pass1<decltype(O)::value, decltype(B)::value><<<g1, kThreads, 0, st>>>(g, cf, u, W, rho0, rho2, S, R,
-                                                                                         partial);
+        constexpr int ORDER = decltype(O)::value, BC = decltype(B)::value;
+        attr = cudaFuncSetAttribute(k_outer_residual<ORDER, BC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)outer_smem_bytes<ORDER>());
+        k_outer_residual<ORDER, BC><<<outer_ctas(g, tg), kOutThreads, outer_smem_bytes<ORDER>(), st>>>(
+            g, make_coef<double>(g, cfg->order), make_outer_int(g, cfg->order), in, R, nullptr, partial, tg, fin);
     };
     using I2 = std::integral_constant<int, 2>;
     using I4 = std::integral_constant<int, 4>;
@@ -193,9 +155,7 @@ extern "C" mg_status mg_residual_norms_noalloc(const mg_config *cfg, const doubl
     } else {
         if (cfg->bc == MG_BC_PERIODIC) launch1(I4(), P()); else launch1(I4(), Rb());
     }
-    k_finalize_sum<5><<<1, 256, 0, st>>>(partial, g1, sc->sums);
-    k_outer_scalars<<<1, 1, 0, st>>>(sc, N, cfg->k_mode == MG_K_INTEGRABILITY, cfg->K * cfg->K,
-                                     cfg->bc == MG_BC_PERIODIC);
+    CK(attr);
     k_noalloc_norms<<<g1, kThreads, 0, st>>>(g, u, R, sc, partial);
     k_finalize_max<4><<<1, 256, 0, st>>>(partial, g1, sc->norms);
     CK(cudaGetLastError());

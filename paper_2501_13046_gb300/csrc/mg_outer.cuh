@@ -1,185 +1,177 @@
-// mg_outer.cuh -- FP64 outer residual of the CTT constraints in two passes.
+// mg_outer.cuh -- FP64 outer residual of the CTT constraints in one fused, tiled pass.
 //
-// On GB300 an FP64 instruction issues at 2 lanes per clock per SM, so this residual is bound by
-// its FP64 instruction count, not by memory.  The mixed term (1/3) d_i d_j W_j of F_W,i costs
-// most: written as the tensor product of first-derivative stencils it takes 16 points and ~20
-// FP64 instructions per (i, j) pair.  Since D_i D_j = D_i o D_j, the same sum is
-//   sum_{j != i} D_i D_j W_j = D_i q_i,   q_i = sum_{j != i} D_j W_j = div W - D_i W_i,
-// so pass A stores q_0, q_1, q_2 and div W at every cell (FP64, from the same boundary values the
-// tensor product uses) and pass B applies one first derivative per row.  Pass B also folds the
-// 1/h factors into the stencil weights.  Pass B takes this path on the interior box (cells
-// whose whole stencil lies inside the box, so the q reads need no ghost value of q); cells of
-// the shell keep the direct tensor-product form.  Both give the discrete operator of the
-// constraints (eq:Ham, eq:Mom in CTT form), differing only in FP64 rounding order.
+// On GB300 an FP64 instruction issues at 2 lanes per clock per SM (conversions to and from FP64
+// too), integer and FP32 instructions at 64 to 128, so a residual written in FP64 arithmetic is
+// bound by its FP64 instruction count: the two-kernel form this replaces spent ~160 of them per
+// cell, 130 on the linear stencils (128^3: 95 us for q, div W, then 589 us; 256^3 Robin 0.6 + 4.8 ms).
+// Here the stencils run on 64-bit integers.  Each CTA brings the planes of (u, W) of its tile into
+// shared memory as fixed-point numbers in units of 2^(E - 56), E the exponent of the largest value
+// the CTA has met so far (one E for u, one for the three W_i: every momentum row and At_ij takes
+// all components).  The stencil weights are small integers (1/12 and 1/h^2 are applied at the
+// end), so sums are exact: |x| < 2^57 units and a 4th-order second difference has weights of
+// total size 64.  A double within 4 binary orders of E is represented exactly, a smaller one to
+// 2^(E - 57), against the 2^(E - 48) an FP64 sum of the same taps rounds by (16 f + 16 f is
+// formed first).  Only the results are converted: Lap u, the three momentum rows, AtAt.  What is
+// left in FP64 is ~33 instructions per cell (powers of psi, the source terms, the block sums).
+//
+// March: 16 x 16 cells per plane, one thread per cell, planes along z through a ring of ORDER + 1
+// slots (2 CTAs per SM).  The mixed term (1/3) d_i d_j W_j uses D_i D_j = D_i o D_j:
+//   row x: D_x B + D_z C,  row y: D_y A + D_z D,  row z: D_z (A + B)
+// with A = D_x W_x, B = D_y W_y, C = D_x W_z, D = D_y W_z formed once per plane; A and B are
+// shared with the neighbouring cells through shared memory, the z history of A + B, C and D stays
+// in the thread's registers.  Boundary values (periodic wrap, Robin, mirror, extrapolation) are
+// filled in when a plane is loaded, in FP64 by the rule of fetch_bc, so every cell takes this path.
+//
+// Values that are NaN or infinite have no fixed-point form: a CTA that meets one finishes its
+// remaining planes with the direct FP64 stencils (outer_cell), which propagate it cell by cell.
+// Fields below 2^-383 (5e-116) everywhere in a tile are held in units of 2^-439.
 #pragma once
 #include "mg_kernels.cuh"
 
 namespace ctt {
 
-// Stencil weights with the grid spacing folded in.
-struct OuterCoef {
-    double c1[3], c2[3];            // D_a f = c1 (f+1 - f-1) - c2 (f+2 - f-2)
-    double k1[3], nk2[3], k0;       // Lap f = k0 f + sum_a k1 (f+1 + f-1) + nk2 (f+2 + f-2)
-    double m1[3][3], nm2[3][3], m0[3];   // row A: Lap W_A + (1/3) D_AA W_A, same form
-    double q1[3], q2[3];            // (1/3) D_A along A
+constexpr int kOutX = 16, kOutY = 16, kOutThreads = kOutX * kOutY;
+constexpr int kOutMaxZ = 16;          // planes per CTA at most
+constexpr int kOutMinExp = 640;       // smallest E (biased): units and their squares stay normal numbers
+constexpr int kOutBadExp = 0x7ff;     // biased exponent of NaN and infinity
+
+template <int ORDER> __host__ __device__ constexpr int outer_w() { return kOutX + ORDER; }        // tile + halo
+template <int ORDER> __host__ __device__ constexpr int outer_plane() { return 4 * outer_w<ORDER>() * outer_w<ORDER>(); }
+template <int ORDER> __host__ __device__ constexpr size_t outer_smem_bytes()
+{   // the ring of planes, then A (tile columns, all rows) and B (all columns, tile rows)
+    return ((size_t)(ORDER + 1) * outer_plane<ORDER>() + 2 * (size_t)kOutX * outer_w<ORDER>()) * sizeof(long long);
+}
+
+// The state and the sources, plain arrays (rho2 may be null: zero).
+struct OuterIn {
+    const double *u, *W, *rho0, *rho2, *S;
 };
 
-// t-th cell (all colours) of the interior box [G, n-G)^3, x fastest; false past the end.
-__device__ __forceinline__ bool interior_cell_all(const Geo &g, int G, unsigned t, int &i, int &j, int &k)
-{
-    const unsigned ix = g.n[0] - 2 * G, iy = g.n[1] - 2 * G, iz = g.n[2] - 2 * G;
-    if ((int)ix <= 0 || (int)iy <= 0 || (int)iz <= 0) return false;
-    const unsigned row = t / ix;
-    if (row >= iy * iz) return false;
-    i = G + (int)(t - row * ix);
-    const unsigned jj = row % iy;
-    j = G + (int)jj;
-    k = G + (int)((row - jj) / iy);
-    return true;
-}
+// Integer weights: with unequal spacings each axis' difference is scaled by its share of the
+// smallest spacing's weight (ratios <= 1 in 64-bit fixed point, the high half of a 64 x 64
+// product); with equal spacings (iso) the shares are 1 and shifts suffice.
+struct OuterInt {
+    int iso;
+    long long wl[3];      // Lap u: (hmin/h_a)^2
+    long long w3[3][3];   // row A: (3 + delta_Aa) (hmin/h_a)^2
+    long long gq[3];      // hmin/h_a, first derivatives inside the mixed term
+    long long gm[3];      // ... outside it, with its 1/6 (order 4) or 1/4 (order 2)
+    long long ga[3];      // ... of At_ij
+    double cu, cm, ca;    // 1/(c hmin^2), a third of it (c = 12 or 1); 1/(c1 hmin) (c1 = 12 or 2)
+};
 
-template <int ORDER, int A, class F>
-__device__ __forceinline__ double d1w(const F &f, double c1, double c2)
+inline OuterInt make_outer_int(const Geo &g, int order)
 {
-    double d = c1 * (ax<A>(f, 1) - ax<A>(f, -1));
-    if constexpr (ORDER == 4) d = fma(-c2, ax<A>(f, 2) - ax<A>(f, -2), d);
-    return d;
-}
-
-template <int ORDER, class F>
-__device__ __forceinline__ double lapw(const F &f, const double k1[3], const double nk2[3], double k0)
-{
-    double s = k0 * f(0, 0, 0);
-    s = fma(k1[0], f(1, 0, 0) + f(-1, 0, 0), s);
-    s = fma(k1[1], f(0, 1, 0) + f(0, -1, 0), s);
-    s = fma(k1[2], f(0, 0, 1) + f(0, 0, -1), s);
-    if constexpr (ORDER == 4) {
-        s = fma(nk2[0], f(2, 0, 0) + f(-2, 0, 0), s);
-        s = fma(nk2[1], f(0, 2, 0) + f(0, -2, 0), s);
-        s = fma(nk2[2], f(0, 0, 2) + f(0, 0, -2), s);
+    OuterInt o;
+    const double hmin = fmin(g.h[0], fmin(g.h[1], g.h[2])), hmax = fmax(g.h[0], fmax(g.h[1], g.h[2]));
+    o.iso = hmax <= hmin * (1.0 + 4.5e-16);   // the same spacing up to the rounding of (hi - lo) / n
+    auto fix = [](long double v, int bits) {  // v 2^bits, at most 2^63 - 1
+        const long double s = ldexpl(v, bits);
+        return s >= 9223372036854775807.0L ? 9223372036854775807LL : (long long)(s + 0.5L);
+    };
+    for (int a = 0; a < 3; ++a) {
+        const long double r = (long double)hmin / (long double)g.h[a];
+        o.wl[a] = fix(r * r, 62);
+        for (int A = 0; A < 3; ++A) o.w3[A][a] = fix((A == a ? 4.0L : 3.0L) * r * r, 60);
+        o.gq[a] = fix(r, 59);
+        o.gm[a] = order == 4 ? fix(r / 6.0L, 64) : fix(r, 62);
+        o.ga[a] = fix(r, 63);
     }
-    return s;
+    o.cu = 1.0 / ((order == 4 ? 12.0 : 1.0) * hmin * hmin);
+    o.cm = o.cu / 3.0;
+    o.ca = 1.0 / ((order == 4 ? 12.0 : 2.0) * hmin);
+    return o;
 }
 
-// Pass A: q_a = div W - D_a W_a (a = 0, 1, 2) and div W, at every cell.
-template <int ORDER, int BC>
-__global__ void __launch_bounds__(256) k_outer_div(Geo g, OuterCoef oc, const double *__restrict__ x,
-                                                   double *__restrict__ D)
+// Launch shape: planes per CTA.  Fewer planes per CTA fill the chip and even out the last wave,
+// each CTA loads ORDER more than it finishes.
+struct OuterGrid {
+    int ntx, nty, zc;
+};
+
+inline OuterGrid outer_grid(const Geo &g)
 {
-    const size_t N = (size_t)g.n[0] * g.n[1] * g.n[2];
-    const int sy = g.n[0], sz = g.n[0] * g.n[1];
-    for (size_t p = blockIdx.x * (size_t)blockDim.x + threadIdx.x; p < N; p += (size_t)gridDim.x * blockDim.x) {
-        const int i = (int)(p % g.n[0]);
-        const size_t rest = p / g.n[0];
-        const int j = (int)(rest % g.n[1]);
-        const int k = (int)(rest / g.n[1]);
-        double h0, h1, h2;
-        if (is_interior(g, i, j, k, halo<ORDER>())) {
-            AccI<double> a1{x + N + p, sy, sz}, a2{x + 2 * N + p, sy, sz}, a3{x + 3 * N + p, sy, sz};
-            h0 = d1w<ORDER, 0>(a1, oc.c1[0], oc.c2[0]);
-            h1 = d1w<ORDER, 1>(a2, oc.c1[1], oc.c2[1]);
-            h2 = d1w<ORDER, 2>(a3, oc.c1[2], oc.c2[2]);
-        } else {
-            AccB<double, BC> a1{x + N, 1, &g, i, j, k}, a2{x + 2 * N, 2, &g, i, j, k}, a3{x + 3 * N, 3, &g, i, j, k};
-            h0 = d1w<ORDER, 0>(a1, oc.c1[0], oc.c2[0]);
-            h1 = d1w<ORDER, 1>(a2, oc.c1[1], oc.c2[1]);
-            h2 = d1w<ORDER, 2>(a3, oc.c1[2], oc.c2[2]);
-        }
-        const double dv = h0 + h1 + h2;
-        D[p] = dv - h0;
-        D[N + p] = dv - h1;
-        D[2 * N + p] = dv - h2;
-        D[3 * N + p] = dv;
-    }
+    constexpr int sms = 152;   // a constant: the workspace (one partial row per CTA) is sized without a device
+    OuterGrid t;
+    t.ntx = (g.n[0] + kOutX - 1) / kOutX;
+    t.nty = (g.n[1] + kOutY - 1) / kOutY;
+    t.zc = kOutMaxZ;
+    while (t.zc > 2 && (long long)t.ntx * t.nty * ((g.n[2] + t.zc - 1) / t.zc) < 6LL * sms) t.zc /= 2;
+    while (t.zc < 4 && (long long)t.ntx * t.nty * ((g.n[2] + t.zc - 1) / t.zc) > 2LL * sms) t.zc *= 2;
+    return t;
 }
 
-// Lap u, AtAt and the momentum operator at a cell from pass A's q, div W (accessors: interior
-// box, or wrapping on periodic boxes, where q and div W are exact at the wrapped cells).
-template <int ORDER, class F>
-__device__ __forceinline__ void outer_cell_qa(const F &u, const F &w0, const F &w1, const F &w2, const F &q0,
-                                              const F &q1, const F &q2, double dv, const OuterCoef &oc, double &lu,
-                                              double &aa, double mom[3], const double *by = nullptr, size_t N = 0)
+inline int outer_ctas(const Geo &g, const OuterGrid &t) { return t.ntx * t.nty * ((g.n[2] + t.zc - 1) / t.zc); }
+
+// ---------------------------------------------------------------- integer stencils
+// taps of one axis around a cell: p1, m1 at distance 1, p2, m2 at 2 (order 4)
+template <int ORDER> struct IAxis { long long m1, p1, m2, p2; };
+
+template <int ORDER>
+__device__ __forceinline__ IAxis<ORDER> itaps(const long long *c, int s)
 {
-    lu = lapw<ORDER>(u, oc.k1, oc.nk2, oc.k0);
-    mom[0] = lapw<ORDER>(w0, oc.m1[0], oc.nm2[0], oc.m0[0]) + d1w<ORDER, 0>(q0, oc.q1[0], oc.q2[0]);
-    mom[1] = lapw<ORDER>(w1, oc.m1[1], oc.nm2[1], oc.m0[1]) + d1w<ORDER, 1>(q1, oc.q1[1], oc.q2[1]);
-    mom[2] = lapw<ORDER>(w2, oc.m1[2], oc.nm2[2], oc.m0[2]) + d1w<ORDER, 2>(q2, oc.q1[2], oc.q2[2]);
-    // At_ab = G_ab + G_ba - (2/3) delta_ab div, G_ab = D_a W_b; the diagonal from pass A
-    const double g00 = dv - q0(0, 0, 0), g11 = dv - q1(0, 0, 0), g22 = dv - q2(0, 0, 0);
-    const double s01 = d1w<ORDER, 0>(w1, oc.c1[0], oc.c2[0]) + d1w<ORDER, 1>(w0, oc.c1[1], oc.c2[1]);
-    const double s02 = d1w<ORDER, 0>(w2, oc.c1[0], oc.c2[0]) + d1w<ORDER, 2>(w0, oc.c1[2], oc.c2[2]);
-    const double s12 = d1w<ORDER, 1>(w2, oc.c1[1], oc.c2[1]) + d1w<ORDER, 2>(w1, oc.c1[2], oc.c2[2]);
-    const double t = (-2.0 / 3.0) * dv;
-    double a00 = fma(2.0, g00, t), a11 = fma(2.0, g11, t), a22 = fma(2.0, g22, t);
-    double b01 = s01, b02 = s02, b12 = s12;
-    if (by) {   // Bowen-York part (by: the cell's first component, stride N)
-        a00 += by[0];
-        a11 += by[N];
-        a22 += by[2 * N];
-        b01 += by[3 * N];
-        b02 += by[4 * N];
-        b12 += by[5 * N];
-    }
-    const double off = fma(b01, b01, fma(b02, b02, b12 * b12));
-    aa = fma(2.0, off, fma(a00, a00, fma(a11, a11, a22 * a22)));
+    if constexpr (ORDER == 4) return {c[-s], c[s], c[-2 * s], c[2 * s]};
+    else return {c[-s], c[s], 0, 0};
+}
+
+// 12 h D f (order 4) or 2 h D f
+template <int ORDER>
+__device__ __forceinline__ long long id1(const IAxis<ORDER> &t)
+{
+    if constexpr (ORDER == 4) return ((t.p1 - t.m1) << 3) - (t.p2 - t.m2);
+    else return t.p1 - t.m1;
+}
+
+// 12 h^2 D2 f (order 4) or h^2 D2 f; k0 = 30 f or 2 f
+template <int ORDER>
+__device__ __forceinline__ long long id2(const IAxis<ORDER> &t, long long k0)
+{
+    if constexpr (ORDER == 4) return ((t.p1 + t.m1) << 4) - (t.p2 + t.m2) - k0;
+    else return t.p1 + t.m1 - k0;
 }
 
 template <int ORDER>
-__device__ __forceinline__ void outer_cell_q(const double *x, const double *D, size_t N, size_t p, int sy, int sz,
-                                             const OuterCoef &oc, double &lu, double &aa, double mom[3],
-                                             const double *by)
+__device__ __forceinline__ long long ik0(long long f)
 {
-    AccI<double> u{x + p, sy, sz}, w0{x + N + p, sy, sz}, w1{x + 2 * N + p, sy, sz}, w2{x + 3 * N + p, sy, sz};
-    AccI<double> q0{D + p, sy, sz}, q1{D + N + p, sy, sz}, q2{D + 2 * N + p, sy, sz};
-    outer_cell_qa<ORDER>(u, w0, w1, w2, q0, q1, q2, D[3 * N + p], oc, lu, aa, mom, by ? by + p : nullptr, N);
+    if constexpr (ORDER == 4) return (f << 5) - (f << 1);
+    else return f << 1;
 }
 
-// Nonlinear terms and outputs at cell p (shared by the interior and shell paths):
-//   R0 = Lap u + (1/8) psi^-7 AtAt + 2 pi (rho0 psi^5 + rho2 psi)
-//   R1..3 = mom_i - 8 pi psi^6 S_i,   R4 = AtAt (pass 2 forms the linearisation coefficient from it,
-//   in the inner solve's precision)
-__device__ __forceinline__ void outer_tail(const Geo &g, int i, int j, int k, size_t p, size_t N, double lu, double aa,
-                                           const double mom[3], const double *x, const double *src, double *R,
-                                           double acc[5])
+// x in units of 2^(E - 56): an FP64 bit pattern of biased exponent <= E, rounded to nearest
+__device__ __forceinline__ long long to_fixed(double x, int E)
 {
-    const double psi = psi_bg(g, i, j, k, p) + x[p];
-    const double rho0 = src[p], rho2 = src[N + p];
-    const double ip = 1.0 / psi;
-    const double p2 = psi * psi, p4 = p2 * p2, p5 = p4 * psi, p6 = p5 * psi;
-    const double ip2 = ip * ip, ip4 = ip2 * ip2, ip7 = ip4 * ip2 * ip;
-    const double nonlin = fma(0.125 * aa, ip7, (2.0 * kPi) * fma(rho0, p5, rho2 * psi));
-    R[p] = lu + nonlin;
-    R[4 * N + p] = aa;
-    acc[0] += nonlin;
-    acc[1] += p5;
-    const double s8 = (8.0 * kPi) * p6;
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        const double s = s8 * src[(2 + a) * N + p];
-        R[(1 + a) * N + p] = mom[a] - s;
-        acc[2 + a] += s;
-    }
+    const int hi = __double2hiint(x), e = (hi >> 20) & 0x7ff;
+    unsigned mh = (unsigned)hi & 0xfffffu;
+    int d = E - e;
+    if (e) mh |= 0x100000u;
+    else --d;   // denormal numbers have the exponent of the smallest normal one
+    const unsigned long long t = (((unsigned long long)mh << 32) | (unsigned)__double2loint(x)) << 4;
+    d = min(d, 62);
+    const unsigned long long v = (t + ((1ULL << d) >> 1)) >> d;
+    return hi < 0 ? -(long long)v : (long long)v;
 }
 
-// Shell cells, out of line so that the interior path keeps its registers.  Periodic boxes: the
-// q form with wrapping accessors; Robin boxes: the direct tensor-product form with boundary
-// values (a ghost value of q is not the Robin value of q).  out = (Lap u, AtAt, mom_0..2).
+__device__ __forceinline__ double pow2_biased(int e) { return __hiloint2double(e << 20, 0); }   // 2^(e - 1023)
+
+// ---------------------------------------------------------------- out-of-line parts
+// Boundary value of field fi (0 = u, 1..3 = W_i) at a cell outside the box.
+template <int BC>
+__device__ __noinline__ double outer_ghost(const double *f, int fi, const Geo &g, int i, int j, int k)
+{
+    return fetch_bc<double, BC>(f, fi, g, i, j, k);
+}
+
+// The direct FP64 form at a cell: out = (Lap u, AtAt, momentum rows).
 template <int ORDER, int BC>
-__device__ __noinline__ void outer_shell_cell(const Geo &g, const Coef<double> &cf, const OuterCoef &oc,
-                                              const double *x, const double *D, int i, int j, int k, double *out)
+__device__ __noinline__ void outer_direct(const Geo &g, const Coef<double> &cf, const double *u, const double *W, int i,
+                                          int j, int k, double *out)
 {
     const size_t N = (size_t)g.n[0] * g.n[1] * g.n[2];
-    AccB<double, BC> a0{x, 0, &g, i, j, k}, a1{x + N, 1, &g, i, j, k}, a2{x + 2 * N, 2, &g, i, j, k},
-        a3{x + 3 * N, 3, &g, i, j, k};
+    const size_t p = (size_t)i + (size_t)g.n[0] * ((size_t)j + (size_t)g.n[1] * k);
+    AccB<double, BC> a0{u, 0, &g, i, j, k}, a1{W, 1, &g, i, j, k}, a2{W + N, 2, &g, i, j, k},
+        a3{W + 2 * N, 3, &g, i, j, k};
     double lu, aa, mom[3];
-    if constexpr (BC == BC_PERIODIC) {
-        AccB<double, BC> q0{D, 0, &g, i, j, k}, q1{D + N, 0, &g, i, j, k}, q2{D + 2 * N, 0, &g, i, j, k};   // periodic
-        const size_t p = (size_t)i + (size_t)g.n[0] * ((size_t)j + (size_t)g.n[1] * k);
-        outer_cell_qa<ORDER>(a0, a1, a2, a3, q0, q1, q2, D[3 * N + p], oc, lu, aa, mom);
-    } else {
-        const size_t p = (size_t)i + (size_t)g.n[0] * ((size_t)j + (size_t)g.n[1] * k);
-        outer_cell<ORDER>(a0, a1, a2, a3, cf, lu, aa, mom, g.by ? g.by + p : nullptr, N);
-    }
+    outer_cell<ORDER>(a0, a1, a2, a3, cf, lu, aa, mom, g.by ? g.by + p : nullptr, N);
     out[0] = lu;
     out[1] = aa;
     out[2] = mom[0];
@@ -187,42 +179,328 @@ __device__ __noinline__ void outer_shell_cell(const Geo &g, const Coef<double> &
     out[4] = mom[2];
 }
 
-// Pass B: residual parts R (5 fields) and block partial sums, as k_outer_pass1.  Blocks
-// [0, rg.nblk_sh) take the shell (tensor-product form), the others the interior box.
-template <int ORDER, int BC>
-__global__ void __launch_bounds__(256, 2) k_outer_pass1q(Geo g, Coef<double> cf, OuterCoef oc,
-                                                      const double *__restrict__ x, const double *__restrict__ D,
-                                                      const double *__restrict__ src, double *__restrict__ R,
-                                                      double *__restrict__ partial, Regions rg, OuterFin fin)
+// Nonlinear terms at cell p, from AtAt: the block sums' terms are added to acc, s = 8 pi psi^6 S_i.
+// Returns (1/8) psi^-7 AtAt + 2 pi (rho0 psi^5 + rho2 psi).
+__device__ __forceinline__ double outer_nonlin(const Geo &g, const OuterIn &in, size_t N, size_t p, int i, int j, int k,
+                                               double aa, double s[3], double acc[5])
 {
+    const double psi = psi_bg(g, i, j, k, p) + in.u[p];
+    const double p2 = psi * psi, p4 = p2 * p2, p5 = p4 * psi, p6 = p5 * psi;
+    const double q = in.rho2 ? fma(in.rho0[p], p5, in.rho2[p] * psi) : in.rho0[p] * p5;
+    const double nonlin = fma(2.0 * kPi, q, (0.125 * aa) * (1.0 / (p6 * psi)));
+    acc[0] += nonlin;
+    acc[1] += p5;
+    const double s8 = (8.0 * kPi) * p6;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        s[a] = s8 * in.S[a * N + p];
+        acc[2 + a] += s[a];
+    }
+    return nonlin;
+}
+
+// ---------------------------------------------------------------- the fused residual
+//   R0 = Lap u + (1/8) psi^-7 AtAt + 2 pi (rho0 psi^5 + rho2 psi)     (F_psi before the K^2 term)
+//   R1..3 = Lap W_i + (1/3) d_i d_j W_j - 8 pi psi^6 S_i                 (F_W before adding m_i)
+//   R4 = AtAt (null: not stored; pass 2 forms the linearisation coefficient from it)
+// and one row of 5 partial sums per CTA; the last CTA finishes the outer scalars when fin.s is set.
+template <int ORDER, int BC>
+__global__ void __launch_bounds__(kOutThreads, 2)
+    k_outer_residual(Geo g, Coef<double> cf, OuterInt oi, OuterIn in, double *__restrict__ R, double *__restrict__ R4,
+                     double *__restrict__ partial, OuterGrid tg, OuterFin fin)
+{
+    constexpr int H = ORDER / 2, W = outer_w<ORDER>(), FE = W * W, PE = outer_plane<ORDER>(), NS = ORDER + 1;
+    constexpr int NE = (PE + kOutThreads - 1) / kOutThreads;   // loaded elements per thread and plane
+    constexpr int NA = (kOutX * W + kOutThreads - 1) / kOutThreads;
+    constexpr int SHU = ORDER == 4 ? 2 : 0, SH3 = ORDER == 4 ? 4 : 0, QS = ORDER == 4 ? 5 : 0;   // pre-shifts of sums
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    long long *ring = reinterpret_cast<long long *>(smem_raw);
+    long long *sA = ring + NS * PE, *sB = sA + kOutX * W;   // A[row][16], B[16 rows][W]
+    __shared__ int sE[2][2];                                // [plane parity][u, W]: largest exponent of a plane
+
     const size_t N = (size_t)g.n[0] * g.n[1] * g.n[2];
-    const int sy = g.n[0], sz = g.n[0] * g.n[1];
-    double acc[5] = {0, 0, 0, 0, 0};
-    int i, j, k;
-    if ((int)blockIdx.x >= rg.nblk_sh) {
-        const unsigned stride = (unsigned)(gridDim.x - rg.nblk_sh) * blockDim.x;
-        for (unsigned t = (blockIdx.x - rg.nblk_sh) * blockDim.x + threadIdx.x; interior_cell_all(g, rg.G, t, i, j, k);
-             t += stride) {
-            const size_t p = (size_t)i + (size_t)sy * j + (size_t)sz * k;
-            double lu, aa, mom[3];
-            outer_cell_q<ORDER>(x, D, N, p, sy, sz, oc, lu, aa, mom, g.by);
-            outer_tail(g, i, j, k, p, N, lu, aa, mom, x, src, R, acc);
+    const int nx = g.n[0], ny = g.n[1], nz = g.n[2], tid = threadIdx.x;
+    const size_t plane = (size_t)nx * ny;
+    int b = blockIdx.x;
+    const int x0 = (b % tg.ntx) * kOutX;
+    b /= tg.ntx;
+    const int y0 = (b % tg.nty) * kOutY;
+    const int z0 = (b / tg.nty) * tg.zc, z1 = min(z0 + tg.zc, nz), NP = z1 - z0 + 2 * H;
+    const int lx = tid & (kOutX - 1), ly = tid / kOutX, i = x0 + lx, j = y0 + ly;
+    const bool act = i < nx && j < ny;
+
+    // loaded elements: in-plane offset of the (wrapped) cell, -1 beyond the halo, -2 a ghost of a box with faces
+    int off[NE];
+#pragma unroll
+    for (int t = 0; t < NE; ++t) {
+        const int e = tid + t * kOutThreads, q = e % FE;
+        int x = x0 - H + q % W, y = y0 - H + q / W;
+        off[t] = -1;
+        if (e < PE && x < nx + H && y < ny + H) {
+            if constexpr (BC == BC_PERIODIC) {
+                x += x < 0 ? nx : (x >= nx ? -nx : 0);
+                y += y < 0 ? ny : (y >= ny ? -ny : 0);
+                off[t] = x + nx * y;
+            } else {
+                off[t] = (x >= 0 && x < nx && y >= 0 && y < ny) ? x + nx * y : -2;
+            }
         }
-    } else {
-        const unsigned stride = (unsigned)rg.nblk_sh * blockDim.x;
-        for (unsigned t = blockIdx.x * blockDim.x + threadIdx.x; shell_cell(g, rg.G, t, i, j, k); t += stride) {
-            const size_t p = (size_t)i + (size_t)sy * j + (size_t)sz * k;
-            double o[5];
-            outer_shell_cell<ORDER, BC>(g, cf, oc, x, D, i, j, k, o);
-            const double mom[3] = {o[2], o[3], o[4]};
-            outer_tail(g, i, j, k, p, N, o[0], o[1], mom, x, src, R, acc);
+    }
+    double raw[NE];
+    auto load = [&](int p) {
+        int z = z0 - H + p;
+        bool zg = false;
+        if constexpr (BC == BC_PERIODIC) z += z < 0 ? nz : (z >= nz ? -nz : 0);
+        else zg = z < 0 || z >= nz;
+#pragma unroll
+        for (int t = 0; t < NE; ++t) {
+            const int f = (tid + t * kOutThreads) / FE;
+            const double *src = f == 0 ? in.u : in.W + (size_t)(f - 1) * N;
+            raw[t] = 0.0;
+            if (off[t] == -1) continue;
+            if (BC != BC_PERIODIC && (zg || off[t] < 0)) {
+                const int q = (tid + t * kOutThreads) % FE;
+                raw[t] = outer_ghost<BC>(src, f, g, x0 - H + q % W, y0 - H + q / W, z);
+            } else {
+                raw[t] = src[(size_t)off[t] + plane * z];
+            }
+        }
+    };
+    auto reduce_exp = [&](int p) {   // into sE[p & 1]
+        int eu = 0, ew = 0;
+#pragma unroll
+        for (int t = 0; t < NE; ++t) {
+            const int e = (__double2hiint(raw[t]) >> 20) & 0x7ff;
+            if (tid + t * kOutThreads < FE) eu = max(eu, e);
+            else ew = max(ew, e);
+        }
+        eu = __reduce_max_sync(0xffffffffu, eu);
+        ew = __reduce_max_sync(0xffffffffu, ew);
+        if ((tid & 31) == 0) {
+            atomicMax(&sE[p & 1][0], eu);
+            atomicMax(&sE[p & 1][1], ew);
+        }
+    };
+    int Eu = kOutMinExp, Ew = kOutMinExp;
+    double wu = 0.0, wm = 0.0, wa = 0.0;   // units of Lap u, of the momentum rows, of At_ij
+    auto set_units = [&]() {
+        wu = oi.cu * pow2_biased(Eu - 56 + SHU);
+        wm = oi.cm * pow2_biased(Ew - 56 + SH3);
+        wa = oi.ca * pow2_biased(Ew - 56);
+    };
+    set_units();
+    long long hs[NS], hc[NS], hd[NS];   // A + B, C, D of the cell, newest plane first
+#pragma unroll
+    for (int k = 0; k < NS; ++k) hs[k] = hc[k] = hd[k] = 0;
+    double acc[5] = {0, 0, 0, 0, 0};
+
+    if (tid < 4) sE[tid >> 1][tid & 1] = 0;
+    load(0);
+    __syncthreads();
+    reduce_exp(0);
+    __syncthreads();
+    int bad = -1;
+    int slot = 0;   // p % NS
+    for (int p = 0; p < NP; ++p) {
+        // phase 0: plane p into the ring in the current units (grown when it holds larger values),
+        // A and B of the centre plane p - H for the tile's neighbours
+        const int eu = sE[p & 1][0], ew = sE[p & 1][1];
+        if (max(eu, ew) == kOutBadExp) { bad = p; break; }
+        if (eu > Eu || ew > Ew) {   // rare: rescale what the ring and the registers hold
+            const int du = min(62, max(0, eu - Eu)), dw = min(62, max(0, ew - Ew));
+            if (p > 0) {
+                for (int e = tid; e < NS * PE; e += kOutThreads) {
+                    const int d = (e % PE) < FE ? du : dw;
+                    ring[e] = (ring[e] + ((1LL << d) >> 1)) >> d;
+                }
+#pragma unroll
+                for (int k = 0; k < NS; ++k) {
+                    hs[k] >>= dw;
+                    hc[k] >>= dw;
+                    hd[k] >>= dw;
+                }
+                __syncthreads();
+            }
+            Eu = max(Eu, eu);
+            Ew = max(Ew, ew);
+            set_units();
+        }
+        {
+            long long *dst = ring + slot * PE;
+#pragma unroll
+            for (int t = 0; t < NE; ++t) {
+                const int e = tid + t * kOutThreads;
+                if (e < PE) dst[e] = to_fixed(raw[t], e < FE ? Eu : Ew);
+            }
+        }
+        if (p + 1 < NP) load(p + 1);
+        const bool full = p >= 2 * H;
+        const int cs = slot >= H ? slot - H : slot - H + NS;   // slot of the centre plane
+        if (full) {
+            const long long *c1 = ring + cs * PE + FE, *c2 = c1 + FE;   // W_x, W_y
+#pragma unroll
+            for (int t = 0; t < NA; ++t) {
+                const int e = tid + t * kOutThreads;
+                if (e < kOutX * W) {
+                    const long long a = id1<ORDER>(itaps<ORDER>(c1 + (e / kOutX) * W + H + e % kOutX, 1));
+                    sA[e] = oi.iso ? a >> QS : __mul64hi(a << (5 - QS), oi.gq[0]);
+                    const long long bb = id1<ORDER>(itaps<ORDER>(c2 + (H + e / W) * W + e % W, W));
+                    sB[e] = oi.iso ? bb >> QS : __mul64hi(bb << (5 - QS), oi.gq[1]);
+                }
+            }
+        }
+        __syncthreads();
+        // phase 1: the new plane's first derivatives, then the centre plane's cell
+        if (tid < 2) sE[p & 1][tid] = 0;
+        const int cell = (ly + H) * W + lx + H;
+        {
+            const long long *q = ring + slot * PE + cell;
+            const long long a = id1<ORDER>(itaps<ORDER>(q + FE, 1)), bb = id1<ORDER>(itaps<ORDER>(q + 2 * FE, W));
+            const long long c = id1<ORDER>(itaps<ORDER>(q + 3 * FE, 1)), d = id1<ORDER>(itaps<ORDER>(q + 3 * FE, W));
+#pragma unroll
+            for (int k = NS - 1; k > 0; --k) {
+                hs[k] = hs[k - 1];
+                hc[k] = hc[k - 1];
+                hd[k] = hd[k - 1];
+            }
+            if (oi.iso) {
+                hs[0] = (a + bb) >> QS;
+                hc[0] = c >> QS;
+                hd[0] = d >> QS;
+            } else {
+                hs[0] = __mul64hi(a << (5 - QS), oi.gq[0]) + __mul64hi(bb << (5 - QS), oi.gq[1]);
+                hc[0] = __mul64hi(c << (5 - QS), oi.gq[0]);
+                hd[0] = __mul64hi(d << (5 - QS), oi.gq[1]);
+            }
+        }
+        if (full && act) {
+            const int k = z0 + p - 2 * H;
+            const size_t P = (size_t)i + (size_t)nx * j + plane * k;
+            const long long *q = ring + cs * PE + cell;
+            // z taps: planes of the ring, as offsets from the centre plane
+            int zo[2 * H];
+#pragma unroll
+            for (int s = 0; s < 2 * H; ++s) {
+                const int dz = s < H ? s - H : s - H + 1;
+                int sl = cs + dz;
+                sl += sl < 0 ? NS : (sl >= NS ? -NS : 0);
+                zo[s] = (sl - cs) * PE;
+            }
+            auto ztaps = [&](const long long *c) -> IAxis<ORDER> {
+                if constexpr (ORDER == 4) return {c[zo[1]], c[zo[2]], c[zo[0]], c[zo[3]]};
+                else return {c[zo[0]], c[zo[1]], 0, 0};
+            };
+            // Lap u
+            long long lu;
+            {
+                const long long k0 = ik0<ORDER>(q[0]);
+                const long long dx = id2<ORDER>(itaps<ORDER>(q, 1), k0), dy = id2<ORDER>(itaps<ORDER>(q, W), k0),
+                                dz = id2<ORDER>(ztaps(q), k0);
+                // (the small constants centre the rounding of the shifts)
+                if (oi.iso) lu = (dx >> SHU) + (dy >> SHU) + (dz >> SHU) + (SHU ? 1 : 0);
+                else
+                    lu = __mul64hi(dx << (2 - SHU), oi.wl[0]) + __mul64hi(dy << (2 - SHU), oi.wl[1]) +
+                         __mul64hi(dz << (2 - SHU), oi.wl[2]) + 1;
+            }
+            // momentum rows, Lap W_A + (1/3) D_AA W_A part, and the first derivatives of W_A
+            long long m[3], g9[3][3];   // g9[a][A] = D_a W_A
+#pragma unroll
+            for (int A = 0; A < 3; ++A) {
+                const long long *w = q + (1 + A) * FE;
+                const long long k0 = ik0<ORDER>(w[0]);
+                const IAxis<ORDER> tx = itaps<ORDER>(w, 1), ty = itaps<ORDER>(w, W), tz = ztaps(w);
+                const long long d0 = id2<ORDER>(tx, k0), d1 = id2<ORDER>(ty, k0), d2 = id2<ORDER>(tz, k0);
+                g9[0][A] = id1<ORDER>(tx);
+                g9[1][A] = id1<ORDER>(ty);
+                g9[2][A] = id1<ORDER>(tz);
+                if (oi.iso) {
+                    const long long e0 = d0 >> SH3, e1 = d1 >> SH3, e2 = d2 >> SH3, s = e0 + e1 + e2;
+                    m[A] = (s << 1) + s + (A == 0 ? e0 : A == 1 ? e1 : e2) + (SH3 ? 5 : 0);
+                } else {
+                    m[A] = __mul64hi(d0 << (4 - SH3), oi.w3[A][0]) + __mul64hi(d1 << (4 - SH3), oi.w3[A][1]) +
+                           __mul64hi(d2 << (4 - SH3), oi.w3[A][2]) + 1;
+                }
+            }
+            // mixed terms
+            {
+                const IAxis<ORDER> bx = itaps<ORDER>(sB + ly * W + lx + H, 1), ay = itaps<ORDER>(sA + (ly + H) * kOutX + lx, kOutX);
+                auto hist = [&](const long long (&h)[NS]) -> IAxis<ORDER> {   // newest plane = centre + H
+                    if constexpr (ORDER == 4) return {h[3], h[1], h[4], h[0]};
+                    else return {h[2], h[0], 0, 0};
+                };
+                const long long xb = id1<ORDER>(bx), ya = id1<ORDER>(ay), zc = id1<ORDER>(hist(hc)),
+                                zd = id1<ORDER>(hist(hd)), zs = id1<ORDER>(hist(hs));
+                if (oi.iso) {
+                    constexpr long long kSixth = 0x2AAAAAAAAAAAAAABLL;   // 2^64 / 6
+                    auto fold = [&](long long v) { return ORDER == 4 ? __mul64hi(v, kSixth) : v >> 2; };
+                    m[0] += fold(xb + zc);
+                    m[1] += fold(ya + zd);
+                    m[2] += fold(zs);
+                } else {
+                    m[0] += __mul64hi(xb, oi.gm[0]) + __mul64hi(zc, oi.gm[2]);
+                    m[1] += __mul64hi(ya, oi.gm[1]) + __mul64hi(zd, oi.gm[2]);
+                    m[2] += __mul64hi(zs, oi.gm[2]);
+                }
+            }
+            // At_ab = D_a W_b + D_b W_a - (2/3) delta_ab div W, then AtAt
+            if (!oi.iso) {
+#pragma unroll
+                for (int a = 0; a < 3; ++a)
+#pragma unroll
+                    for (int A = 0; A < 3; ++A) g9[a][A] = __mul64hi(g9[a][A] << 1, oi.ga[a]);
+            }
+            constexpr long long kThird = 0x5555555555555555LL;   // 2^64 / 3
+            const long long third = __mul64hi(g9[0][0] + g9[1][1] + g9[2][2], kThird);
+            long long at[6] = {(g9[0][0] - third) << 1, (g9[1][1] - third) << 1, (g9[2][2] - third) << 1,
+                               g9[0][1] + g9[1][0], g9[0][2] + g9[2][0], g9[1][2] + g9[2][1]};
+            double aa;
+            if (g.by) {   // with the punctures' analytic part, in FP64
+                const double *by = g.by + P;
+                double v[6];
+#pragma unroll
+                for (int c = 0; c < 6; ++c) v[c] = fma((double)at[c], wa, by[c * N]);
+                aa = fma(2.0, fma(v[3], v[3], fma(v[4], v[4], v[5] * v[5])), fma(v[0], v[0], fma(v[1], v[1], v[2] * v[2])));
+            } else {      // squares of the entries shifted up to 61 bits, high halves of the products
+                long long any = 0;
+#pragma unroll
+                for (int c = 0; c < 6; ++c) any |= at[c] ^ (at[c] >> 63);
+                const int sh = __clzll(any) - 3;
+#pragma unroll
+                for (int c = 0; c < 6; ++c) {
+                    const long long v = sh < 0 ? at[c] >> -sh : at[c] << sh;
+                    at[c] = __mul64hi(v, v);
+                }
+                const long long sq = at[0] + at[1] + at[2] + ((at[3] + at[4] + at[5]) << 1);
+                const double w2 = wa * pow2_biased(1023 + 32 - sh);
+                aa = sq == 0 ? 0.0 : (double)sq * (w2 * w2);
+            }
+            double s[3];
+            const double nonlin = outer_nonlin(g, in, N, P, i, j, k, aa, s, acc);
+            R[P] = fma((double)lu, wu, nonlin);
+#pragma unroll
+            for (int A = 0; A < 3; ++A) R[(1 + A) * N + P] = fma((double)m[A], wm, -s[A]);
+            if (R4) R4[P] = aa;
+        }
+        if (p + 1 < NP) reduce_exp(p + 1);
+        __syncthreads();
+        slot = slot + 1 == NS ? 0 : slot + 1;
+    }
+    if (bad >= 0 && act) {   // a NaN or an infinity: the planes not finished yet, directly
+        for (int k = z0 + max(0, bad - 2 * H); k < z1; ++k) {
+            const size_t P = (size_t)i + (size_t)nx * j + plane * k;
+            double o[5], s[3];
+            outer_direct<ORDER, BC>(g, cf, in.u, in.W, i, j, k, o);
+            const double nonlin = outer_nonlin(g, in, N, P, i, j, k, o[1], s, acc);
+            R[P] = o[0] + nonlin;
+            for (int A = 0; A < 3; ++A) R[(1 + A) * N + P] = o[2 + A] - s[A];
+            if (R4) R4[P] = o[1];
         }
     }
     double r[5];
     block_sum<5>(acc, r);
-    if (threadIdx.x == 0)
+    if (tid == 0)
         for (int a = 0; a < 5; ++a) partial[blockIdx.x * 5 + a] = r[a];
-    if (fin.s && finalize_last<5, false>(partial, gridDim.x, fin.s->sums, &fin.s->ticket[0]) && threadIdx.x == 0)
+    if (fin.s && finalize_last<5, false>(partial, gridDim.x, fin.s->sums, &fin.s->ticket[0]) && tid == 0)
         outer_scalars(fin.s, N, fin.kmode_integrability, fin.K2_fixed, fin.periodic);
 }
 
