@@ -298,7 +298,7 @@ mg_status mg_fp64_fma_rate(struct mg_ctx *ctx, int reps, double *tflops);
  *   K2          host pointer or NULL: the K^2 used (integrability value on periodic boxes).
  *   cuda_stream stream for all work (NULL = legacy default stream); the call synchronises it.
  *
- * Scratch: one file-scope device array of 8.47 MB, which every GPU that loads the library
+ * Scratch: one file-scope device array of 8.55 MB, which every GPU that loads the library
  * holds until the process exits.  The first call on a device looks up that device's address of
  * the array (with the device current) and caches it: that first call on each device should come
  * before any stream capture begins.  All calls share the array and it keeps the last call's contents;

@@ -15,9 +15,10 @@ namespace {
 
 constexpr size_t kNoallocMaxCells = 64 * 64 * 64;                 // 262,144 cells
 constexpr size_t kNoallocR = 4 * kNoallocMaxCells;                // pass-1 output, 4 FP64 fields
-constexpr size_t kNoallocPartials = (size_t)kRedBlocks * 8;       // block partials (5 per CTA of the residual, 4 of the norms)
+constexpr size_t kNoallocPartials = 4096 * 5;                      // block partials: 5 per CTA of the residual
 constexpr size_t kNoallocScalars = 64;                            // >= sizeof(Scalars) / 8
-constexpr size_t kNoallocDoubles = kNoallocR + kNoallocPartials + kNoallocScalars;   // 8.47 MB
+constexpr size_t kNoallocDoubles = kNoallocR + kNoallocPartials + kNoallocScalars;   // 8.55 MB
+static_assert(kNoallocPartials >= (size_t)kRedBlocks * 4, "the norms' partials fit too");
 static_assert(sizeof(Scalars) <= kNoallocScalars * sizeof(double), "scalar slot too small");
 
 static __device__ __align__(256) double g_noalloc_scratch[kNoallocDoubles];
@@ -134,7 +135,7 @@ extern "C" mg_status mg_residual_norms_noalloc(const mg_config *cfg, const doubl
     CK(cudaMemsetAsync(sc, 0, sizeof(Scalars), st));
     const int g1 = grid_for(N, kRedBlocks);
     const OuterGrid tg = outer_grid(g);
-    if ((size_t)outer_ctas(g, tg) * 5 > kNoallocPartials)   // (at most 1824 CTAs on 262144 cells)
+    if ((size_t)outer_ctas(g, tg) * 5 > kNoallocPartials)   // (at most 3641 CTAs on 262144 cells: 3 x 29127 x 3)
         return fail(MG_ERR_INVALID_ARG, "mg_residual_norms_noalloc: too many tiles for the static scratch");
     const OuterIn in{u, W, rho0, rho2, S};
     const OuterFin fin{sc, cfg->k_mode == MG_K_INTEGRABILITY, cfg->bc == MG_BC_PERIODIC, cfg->K * cfg->K};
