@@ -295,8 +295,7 @@ __global__ void k_fill_value(void *p, size_t n, int tb, double v)
 mg_status project_gauge(mg_ctx *x)
 {
     if (x->cfg.bc != MG_BC_PERIODIC) return MG_OK;
-    int g = grid_for(x->N, kRedBlocks);
-    k_sum4<double><<<g, kThreads, 0, x->stream>>>(x->X, x->N, x->partial, x->scal->emean, &x->scal->ticket[2]);
+    k_sum4<double><<<grid_for((x->N + 1) / 2, kSumBlocks), kThreads, 0, x->stream>>>(x->X, x->N, x->partial, x->scal->emean, &x->scal->ticket[2]);
     k_sub_mean4<double><<<grid_for(x->N), kThreads, 0, x->stream>>>(x->X, x->N, x->scal->emean);
     CK(cudaGetLastError());
     return MG_OK;

@@ -235,19 +235,31 @@ mg_status enqueue_outer_pass1(mg_ctx *x, const OuterFin &fin)
     return MG_OK;
 }
 
+// The scalars go to the host, unless a device-side controller reads them (device-paced batch).
+inline mg_status enqueue_read_scalars(mg_ctx *x)
+{
+    if (!x->device_paced) CK(cudaMemcpyAsync(x->host_scal, x->scal, sizeof(Scalars), cudaMemcpyDeviceToHost, x->stream));
+    return MG_OK;
+}
+
 // Outer residual.  HM != nullptr: write H, M instead of the inner rhs/coefficient.
 template <typename T, int ORDER, int BC>
 mg_status enqueue_residual(mg_ctx *x, double *HM)
 {
     LevelBufs &L0 = x->lev[0];
     CKS(enqueue_outer_pass1<T, ORDER, BC>(x, outer_fin(x)));
-    int g1 = grid_for(x->N, kRedBlocks);
-    k_outer_pass2<T><<<g1, kThreads, 0, x->stream>>>(L0.geo, x->X, x->R, x->SRC, x->scal, (T *)L0.f, (T *)L0.c, HM,
-                                                     x->partial, L0.split, 1);
+    if constexpr (sizeof(T) == 4) {
+        if (!HM && L0.split) {
+            k_outer_pass2_pairs<<<grid_for(x->N / 2, kRedBlocks), kThreads, 0, x->stream>>>(
+                L0.geo, x->X, x->R, x->SRC, x->scal, (T *)L0.f, (T *)L0.c, x->partial);
+            CK(cudaGetLastError());
+            return enqueue_read_scalars(x);
+        }
+    }
+    k_outer_pass2<T><<<grid_for(x->N, kRedBlocks), kThreads, 0, x->stream>>>(
+        L0.geo, x->X, x->R, x->SRC, x->scal, (T *)L0.f, (T *)L0.c, HM, x->partial, L0.split);
     CK(cudaGetLastError());
-    // the scalars go to the host, unless a device-side controller reads them (device-paced batch)
-    if (!x->device_paced) CK(cudaMemcpyAsync(x->host_scal, x->scal, sizeof(Scalars), cudaMemcpyDeviceToHost, x->stream));
-    return MG_OK;
+    return enqueue_read_scalars(x);
 }
 
 // Shared memory of a one-CTA Gauss-Jordan inversion of order m in type C (0: the matrix stays in
@@ -322,7 +334,7 @@ mg_status enqueue_iteration(mg_ctx *x)
         L0.f = f;
         CKS(st);
         CK(cudaMemcpyAsync(x->zbuf, L0.cur(), 4 * x->N * sizeof(T), cudaMemcpyDeviceToDevice, x->stream));
-        k_sum4<T><<<grid_for(x->N, kRedBlocks), kThreads, 0, x->stream>>>((const T *)x->zbuf, x->N, x->partial,
+        k_sum4<T><<<grid_for((x->N + 3) / 4, kSumBlocks), kThreads, 0, x->stream>>>((const T *)x->zbuf, x->N, x->partial,
                                                                         x->scal->zmean, &x->scal->ticket[2]);
         CK(cudaGetLastError());
         return MG_OK;
@@ -330,14 +342,15 @@ mg_status enqueue_iteration(mg_ctx *x)
     for (int cyc = 0; cyc < x->cfg.inner_cycles; ++cyc) CKS(enqueue_vcycle<T, ORDER, BC>(x, cyc == 0));
     int periodic = x->cfg.bc == MG_BC_PERIODIC;
     if (periodic) {
-        int g = grid_for(x->N, kRedBlocks);
-        k_sum4<T><<<g, kThreads, 0, x->stream>>>((const T *)L0.cur(), x->N, x->partial, x->scal->emean,
+        k_sum4<T><<<grid_for((x->N + 3) / 4, kSumBlocks), kThreads, 0, x->stream>>>((const T *)L0.cur(), x->N, x->partial, x->scal->emean,
                                                  &x->scal->ticket[2]);
     }
     // the size of the update is reduced only for the per-field stopping test (field_tol > 0)
     const bool sized = x->cfg.field_tol > 0.0;
-    k_update<T><<<sized ? grid_for(x->N, kRedBlocks) : grid_for(x->N), kThreads, 0, x->stream>>>(
-        L0.geo, x->X, (const T *)L0.cur(), x->N, periodic ? x->scal->emean : nullptr, L0.split, x->partial,
+    const size_t items = L0.split ? x->N / 2 : x->N;
+    auto update = sized ? (L0.split ? k_update<T, 1, 1> : k_update<T, 0, 1>) : (L0.split ? k_update<T, 1, 0> : k_update<T, 0, 0>);
+    update<<<sized ? grid_for(items, kRedBlocks) : grid_for(items), kThreads, 0, x->stream>>>(
+        L0.geo, x->X, (const T *)L0.cur(), x->N, periodic ? x->scal->emean : nullptr, x->partial,
         sized ? x->scal : nullptr, x->zbuf && periodic ? (const T *)x->zbuf : nullptr, x->scal->zmean);
     CK(cudaGetLastError());
     return enqueue_residual<T, ORDER, BC>(x, nullptr);

@@ -310,7 +310,7 @@ __global__ void __launch_bounds__(256) k_fill_robin_table(Geo g, double *__restr
     }
 }
 
-__device__ __forceinline__ double psi_background(const Geo &g, int i, int j, int k)
+static __device__ __noinline__ double psi_background(const Geo &g, int i, int j, int k)
 {
     double v = 1.0;
     for (int p = 0; p < g.npunct; ++p) {
@@ -323,10 +323,12 @@ __device__ __forceinline__ double psi_background(const Geo &g, int i, int j, int
 }
 
 // psi_background at cell p = (i, j, k): the stored table when there is one (a FP64 square root and
-// division per puncture and cell cost more than the 8-byte read), else formed in place.
+// division per puncture and cell cost more than the 8-byte read), 1 without punctures, else formed in
+// place (out of line: only a caller's own state with punctures, mg_residual_norms_noalloc, gets there).
 __device__ __forceinline__ double psi_bg(const Geo &g, int i, int j, int k, size_t p)
 {
-    return g.psibg ? g.psibg[p] : psi_background(g, i, j, k);
+    if (g.psibg) return g.psibg[p];
+    return g.npunct == 0 ? 1.0 : psi_background(g, i, j, k);
 }
 
 static __global__ void __launch_bounds__(256) k_fill_psibg(Geo g, double *__restrict__ pb)
@@ -934,24 +936,29 @@ __device__ __forceinline__ void block_sum(double (&v)[NV], double *out /* per bl
     __syncthreads();
 }
 
+// Maxima of values >= 0 (no NaN), compared as bit patterns: an FP64 maximum per value, warp and step
+// would cost a block ~5000 cycles of the FP64 pipe.
 template <int NV>
 __device__ __forceinline__ void block_max(double (&v)[NV], double *out)
 {
-    __shared__ double sh[32][NV];
+    __shared__ unsigned long long sh[32][NV];
+    auto larger = [](unsigned long long a, unsigned long long b) { return a > b ? a : b; };
+    const int w = threadIdx.x >> 5, l = threadIdx.x & 31, nw = (blockDim.x + 31) >> 5;
+    unsigned long long m[NV];
 #pragma unroll
-    for (int a = 0; a < NV; ++a)
-        for (int o = 16; o > 0; o >>= 1) v[a] = fmax(v[a], __shfl_down_sync(0xffffffffu, v[a], o));
-    int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+    for (int a = 0; a < NV; ++a) {
+        m[a] = (unsigned long long)__double_as_longlong(v[a]);
+        for (int o = 16; o > 0; o >>= 1) m[a] = larger(m[a], __shfl_down_sync(0xffffffffu, m[a], o));
+    }
     if (l == 0)
-        for (int a = 0; a < NV; ++a) sh[w][a] = v[a];
+        for (int a = 0; a < NV; ++a) sh[w][a] = m[a];
     __syncthreads();
     if (w == 0) {
-        int nw = (blockDim.x + 31) >> 5;
 #pragma unroll
         for (int a = 0; a < NV; ++a) {
-            double s = l < nw ? sh[l][a] : 0.0;
-            for (int o = 16; o > 0; o >>= 1) s = fmax(s, __shfl_down_sync(0xffffffffu, s, o));
-            if (l == 0) out[a] = s;
+            unsigned long long s = l < nw ? sh[l][a] : 0ULL;
+            for (int o = 16; o > 0; o >>= 1) s = larger(s, __shfl_down_sync(0xffffffffu, s, o));
+            if (l == 0) out[a] = __longlong_as_double((long long)s);
         }
     }
     __syncthreads();
@@ -977,7 +984,8 @@ __device__ __forceinline__ bool finalize_last(const double *partial, int nblocks
 #pragma unroll
         for (int a = 0; a < NV; ++a) {
             const double p = __ldcg(partial + b * NV + a);
-            v[a] = MAX ? fmax(v[a], p) : v[a] + p;
+            if constexpr (MAX) v[a] = __double_as_longlong(p) > __double_as_longlong(v[a]) ? p : v[a];   // (values >= 0)
+            else v[a] += p;
         }
     double r[NV];
     if constexpr (MAX) block_max<NV>(v, r);
@@ -987,8 +995,57 @@ __device__ __forceinline__ bool finalize_last(const double *partial, int nblocks
     return true;
 }
 
-// |x| with NaN mapped to +inf, so that a max-reduction cannot hide it
-__device__ __forceinline__ double absnan(double x) { return (x == x) ? fabs(x) : __longlong_as_double(0x7ff0000000000000ULL); }
+// FP64 compares, conversions and divisions issue at 2 lanes per clock per SM on this GPU; the passes over
+// whole fields below form them with integer instructions (64 to 128 lanes per clock).
+
+// Running maximum of |x| on bit patterns (ordered like the values; a NaN lies above infinity, so it cannot hide).
+__device__ __forceinline__ void max_abs(unsigned long long &m, double x)
+{
+    const unsigned long long b = (unsigned long long)__double_as_longlong(x) & 0x7fffffffffffffffULL;
+    m = b > m ? b : m;
+}
+// ... and its value, a NaN as +inf
+__device__ __forceinline__ double max_value(unsigned long long m)
+{
+    return __longlong_as_double((long long)(m > 0x7ff0000000000000ULL ? 0x7ff0000000000000ULL : m));
+}
+
+// The conversion instructions, out of line: inlined, the compiler would run them for every value and select.
+static __device__ __noinline__ double cvt_f64_any(float x) { return (double)x; }
+static __device__ __noinline__ float cvt_f32_any(double x) { return (float)x; }
+
+// (double)x, exact: normal numbers and zeros by their bits, the rest by the conversion instruction.
+__device__ __forceinline__ double to_f64(float x)
+{
+    const unsigned u = __float_as_uint(x), mag = u & 0x7fffffffu;
+    if (mag - 0x00800000u >= 0x7f000000u && mag != 0) return cvt_f64_any(x);   // denormal, infinite, NaN
+    const unsigned hi = mag ? (mag >> 3) + 0x38000000u : 0u;
+    return __hiloint2double((int)(hi | (u & 0x80000000u)), (int)(u << 29));
+}
+__device__ __forceinline__ double to_f64(double x) { return x; }
+
+// (float)x, rounded to nearest even: results in the normal range and zeros by their bits.
+__device__ __forceinline__ float to_f32(double x)
+{
+    const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x), mag = hi & 0x7fffffffu;
+    const unsigned h = mag - (896u << 20);
+    if (h - 0x00100000u >= 0x0fe00000u && (mag | lo) != 0) return cvt_f32_any(x);   // outside 2^-126 .. 2^128
+    unsigned v = __funnelshift_l(lo, h, 3);
+    v += (lo & 0x1fffffffu) + (v & 1u) > 0x10000000u ? 1u : 0u;
+    return __uint_as_float(((mag | lo) ? v : 0u) | (hi & 0x80000000u));
+}
+
+// 1/x to FP64 rounding: the hardware's approximate reciprocal y and one third-order step
+// y + y (r + r^2), r = 1 - x y (the geometric series of 1/(1 - r)), without the branches of the
+// IEEE division; where x y is not near 1 (x = 0, infinite or next to overflow) y is the limit itself.
+__device__ __forceinline__ double recip_f64(double x)
+{
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double r = fma(-x, y, 1.0);
+    const double t = fma(y, fma(r, r, r), y);
+    return ((__double2hiint(r) >> 20) & 0x7ff) < 1023 - 10 ? t : y;   // |r| < 2^-10, not NaN
+}
 
 // Scalars shared by the outer iteration (device memory).
 struct Scalars {
@@ -1072,30 +1129,78 @@ __global__ void k_finalize_max(const double *__restrict__ partial, int nblocks, 
 }
 
 // Sums of 4 contiguous fields (block partials); with means != nullptr the last block also forms
-// means[a] = sum_a / N (ticket: its finalize_last counter).
+// means[a] = sum_a / N (ticket: its finalize_last counter).  Fields of a multiple of 4 cells (every
+// grid with more than one level) are read 16 bytes at a time.  128^3 FP32: 35 -> 9 us.
+constexpr int kSumBlocks = 152 * 2;
+
+// s + b as an unevaluated pair hi + lo of floats, exact (Knuth's two-sum; the rounding error of every addition
+// is carried in lo)
+__device__ __forceinline__ void two_sum_add(float &hi, float &lo, float b)
+{
+    const float s = __fadd_rn(hi, b);
+    const float bv = __fsub_rn(s, hi);
+    const float err = __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bv)), __fsub_rn(b, bv));
+    hi = s;
+    lo = __fadd_rn(lo, err);
+}
+
 template <typename T>
 __global__ void __launch_bounds__(256) k_sum4(const T *__restrict__ x, size_t N, double *__restrict__ partial,
                                               double *__restrict__ means, unsigned int *ticket)
 {
+    __shared__ double sw[32][4];
     double v[4] = {0, 0, 0, 0};
-    if constexpr (sizeof(T) == 4) {
-        // each thread's sum as an unevaluated pair hi + lo of floats, kept exact by Knuth's
-        // two-sum (the rounding error of every addition is carried in lo), then one FP64 sum
-        float hi[4] = {0, 0, 0, 0}, lo[4] = {0, 0, 0, 0};
-        for (size_t p = blockIdx.x * (size_t)blockDim.x + threadIdx.x; p < N; p += (size_t)gridDim.x * blockDim.x)
+    const size_t t0 = blockIdx.x * (size_t)blockDim.x + threadIdx.x, stride = (size_t)gridDim.x * blockDim.x;
+    if constexpr (sizeof(T) == 4) {   // each thread's sums as float pairs, then one FP64 sum each
+        float hi[4][2] = {}, lo[4][2] = {};
+        if (N % 4 == 0) {
+            for (size_t p = t0; p < N / 4; p += stride) {
+                float4 b[4];
+#pragma unroll
+                for (int a = 0; a < 4; ++a) b[a] = reinterpret_cast<const float4 *>(x + a * N)[p];
+#pragma unroll
+                for (int a = 0; a < 4; ++a) {
+                    two_sum_add(hi[a][0], lo[a][0], b[a].x);
+                    two_sum_add(hi[a][1], lo[a][1], b[a].y);
+                    two_sum_add(hi[a][0], lo[a][0], b[a].z);
+                    two_sum_add(hi[a][1], lo[a][1], b[a].w);
+                }
+            }
+        } else {
+            for (size_t p = t0; p < N; p += stride)
+#pragma unroll
+                for (int a = 0; a < 4; ++a) two_sum_add(hi[a][0], lo[a][0], (float)x[a * N + p]);
+        }
+        // the pairs of a warp are added as pairs too: one FP64 conversion per warp, not per thread
+#pragma unroll
+        for (int a = 0; a < 4; ++a) {
+            two_sum_add(hi[a][0], lo[a][0], hi[a][1]);
+            lo[a][0] += lo[a][1];
+            for (int o = 16; o > 0; o >>= 1) {
+                const float h = __shfl_xor_sync(0xffffffffu, hi[a][0], o), l = __shfl_xor_sync(0xffffffffu, lo[a][0], o);
+                two_sum_add(hi[a][0], lo[a][0], h);
+                lo[a][0] += l;
+            }
+            if ((threadIdx.x & 31) == 0) sw[threadIdx.x >> 5][a] = (double)hi[a][0] + (double)lo[a][0];
+        }
+        __syncthreads();
+        if (threadIdx.x < 4) {
+            double t = 0.0;
+            for (int w = 0; w < (int)blockDim.x / 32; ++w) t += sw[w][threadIdx.x];
+            partial[blockIdx.x * 4 + threadIdx.x] = t;
+        }
+        if (means && finalize_last<4, false>(partial, gridDim.x, means, ticket) && threadIdx.x == 0)
+            for (int a = 0; a < 4; ++a) means[a] = means[a] / (double)N;
+        return;
+    } else if (N % 4 == 0) {
+        for (size_t p = t0; p < N / 2; p += stride)
 #pragma unroll
             for (int a = 0; a < 4; ++a) {
-                const float b = (float)x[a * N + p];
-                const float s = __fadd_rn(hi[a], b);
-                const float bv = __fsub_rn(s, hi[a]);
-                const float err = __fadd_rn(__fsub_rn(hi[a], __fsub_rn(s, bv)), __fsub_rn(b, bv));
-                hi[a] = s;
-                lo[a] = __fadd_rn(lo[a], err);
+                const double2 b = reinterpret_cast<const double2 *>(x + a * N)[p];
+                v[a] += b.x + b.y;
             }
-#pragma unroll
-        for (int a = 0; a < 4; ++a) v[a] = (double)hi[a] + (double)lo[a];
     } else {
-        for (size_t p = blockIdx.x * (size_t)blockDim.x + threadIdx.x; p < N; p += (size_t)gridDim.x * blockDim.x)
+        for (size_t p = t0; p < N; p += stride)
 #pragma unroll
             for (int a = 0; a < 4; ++a) v[a] += (double)x[a * N + p];
     }
@@ -1120,41 +1225,77 @@ __global__ void __launch_bounds__(256) k_sub_mean4(T *__restrict__ x, size_t N, 
 }
 
 // State update u += e - <e>, W_i += e_i - <e_i> (means only on periodic boxes); e is stored in
-// the finest level's layout (colour-split when split != 0).  With s set, the last block also
+// the finest level's layout (colour-split when split != 0).  With SIZED, the last block also
 // leaves the size of the update in s->change: per field the largest applied correction and the
 // largest |psi|, |W_i| after it (psi = background + u), for the per-field stopping test.
 // Launched on at most kRedBlocks blocks (partial holds 8 values per block).
-template <typename T>
-__global__ void __launch_bounds__(256) k_update(Geo g, double *__restrict__ x, const T *__restrict__ e, size_t N,
-                                                const double *__restrict__ means, int split,
-                                                double *__restrict__ partial, Scalars *s, const T *__restrict__ z,
-                                                const double *__restrict__ zmean)
+// Split levels take the two cells of an x pair per thread (16-byte accesses of x, one value of each colour
+// half); with the conversions by bits two FP64 additions per value are left (one without means).
+template <typename T, int SPLIT, int SIZED>
+__global__ void __launch_bounds__(256, SIZED ? 2 : 4) k_update(Geo g, double *__restrict__ x, const T *__restrict__ e, size_t N,
+                                                const double *__restrict__ means, double *__restrict__ partial,
+                                                Scalars *s, const T *__restrict__ z, const double *__restrict__ zmean)
 {
     // z (k2_newton): the psi correction's mean is removed along z, scaled so that the mean goes
     const double zr = z ? means[0] / zmean[0] : 0.0;
     double m[4];
 #pragma unroll
     for (int a = 0; a < 4; ++a) m[a] = means ? means[a] : 0.0;
-    double mx[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+    unsigned long long mx[8] = {0, 0, 0, 0, 0, 0, 0, 0};
     const unsigned nx = (unsigned)g.n[0], ny = (unsigned)g.n[1];   // grids hold < 2^31 cells
-    for (size_t p = blockIdx.x * (size_t)blockDim.x + threadIdx.x; p < N; p += (size_t)gridDim.x * blockDim.x) {
-        const unsigned pu = (unsigned)p, rest = pu / nx;
-        const unsigned i = pu - rest * nx, j = rest % ny, k = rest / ny;
-        const size_t q = split ? (((i + j + k) & 1) ? N / 2 : 0) + (p >> 1) : p;
+    // the applied correction, from e's value at storage index q; the field's new value v is recorded for the stopping test
+    auto delta = [&](int a, T ev, size_t q) {
+        const double d = to_f64(ev);
+        if (z && a == 0) return d - zr * to_f64(z[q]);
+        return means ? d - m[a] : d;
+    };
+    auto record = [&](int a, double d, double v, int i, int j, int k, size_t p) {
+        max_abs(mx[a], d);
+        max_abs(mx[4 + a], a == 0 ? psi_bg(g, i, j, k, p) + v : v);
+    };
+    const size_t t0 = blockIdx.x * (size_t)blockDim.x + threadIdx.x, stride = (size_t)gridDim.x * blockDim.x;
+    if constexpr (SPLIT) {
+        const unsigned nxh = nx >> 1;
+        for (size_t pm = t0; pm < N / 2; pm += stride) {
+            const unsigned row = (unsigned)pm / nxh, i = 2 * ((unsigned)pm - row * nxh), j = row % ny, k = row / ny;
+            const size_t c = (j + k) & 1;   // colour of the even-x cell
+            const size_t q0 = pm + (c ? N / 2 : 0), q1 = pm + (c ? 0 : N / 2);
+            double2 v[4];
+            T e0[4], e1[4];
 #pragma unroll
-        for (int a = 0; a < 4; ++a) {
-            const double d = (z && a == 0) ? (double)e[q] - zr * (double)z[q] : (double)e[a * N + q] - m[a];
-            const double v = x[a * N + p] + d;
-            x[a * N + p] = v;
-            if (s) {
-                mx[a] = fmax(mx[a], absnan(d));
-                mx[4 + a] = fmax(mx[4 + a], absnan(a == 0 ? psi_bg(g, (int)i, (int)j, (int)k, p) + v : v));
+            for (int a = 0; a < 4; ++a) {   // every load before the first store
+                v[a] = reinterpret_cast<const double2 *>(x + a * N)[pm];
+                e0[a] = e[a * N + q0];
+                e1[a] = e[a * N + q1];
+            }
+#pragma unroll
+            for (int a = 0; a < 4; ++a) {
+                const double d0 = delta(a, e0[a], q0), d1 = delta(a, e1[a], q1);
+                v[a].x += d0;
+                v[a].y += d1;
+                reinterpret_cast<double2 *>(x + a * N)[pm] = v[a];
+                if (SIZED) {
+                    record(a, d0, v[a].x, (int)i, (int)j, (int)k, 2 * pm);
+                    record(a, d1, v[a].y, (int)i + 1, (int)j, (int)k, 2 * pm + 1);
+                }
+            }
+        }
+    } else {
+        for (size_t p = t0; p < N; p += stride) {
+            const unsigned rest = (unsigned)p / nx, i = (unsigned)p - rest * nx, j = rest % ny, k = rest / ny;
+#pragma unroll
+            for (int a = 0; a < 4; ++a) {
+                const double d = delta(a, e[a * N + p], p), v = x[a * N + p] + d;
+                x[a * N + p] = v;
+                if (SIZED) record(a, d, v, (int)i, (int)j, (int)k, p);
             }
         }
     }
-    if (!s) return;
-    double r[8];
-    block_max<8>(mx, r);
+    if constexpr (!SIZED) return;
+    double mv[8], r[8];
+#pragma unroll
+    for (int a = 0; a < 8; ++a) mv[a] = max_value(mx[a]);
+    block_max<8>(mv, r);
     if (threadIdx.x == 0)
         for (int a = 0; a < 8; ++a) partial[blockIdx.x * 8 + a] = r[a];
     finalize_last<8, true>(partial, gridDim.x, s->change, &s->ticket[3]);
@@ -1208,25 +1349,87 @@ __device__ __forceinline__ void outer_cell(const F &u, const F &w0, const F &w1,
 // Pass 2: final residuals, norm partials, inner right-hand side and coefficients in T:
 //   f = (-psi^-5 F_psi, -F_W,i),  a = psi^-5,  b = psi^-5 c,  c = dF_psi/du.
 // F_psi = R0 - (K^2/12) psi^5 and F_W,i = R_i + m_i are always formed in FP64: these are the
-// differences of nearly equal terms.  With an FP32 inner solve (T = float) and no field output,
+// differences of nearly equal terms.  With an FP32 inner solve (T = float, k_outer_pass2_pairs),
 // the later products (the psi^-5, psi^-6 scalings of H and M, the inner data) are formed in FP32:
 // each is a product of already-accurate factors, so the norms keep 7 significant digits and the
 // FP64 ALU, at 2 lanes per clock per SM on this GPU, is spared the division and powers.
-// Optionally (HM != nullptr) writes H and M (4 FP64 fields, FP64 throughout) instead.
+// Optionally (HM != nullptr) k_outer_pass2 writes H and M (4 FP64 fields, FP64 throughout) instead.
 __device__ __forceinline__ float absnanf(float x) { return (x == x) ? fabsf(x) : __int_as_float(0x7f800000); }
+
+// The FP32 inner solve's form, on a colour-split finest level: the two cells of an x pair per thread,
+// 16-byte loads, conversions to FP32 by bits (8 FP64 instructions per cell are left of 17; 5 on boxes
+// without momentum-source means).  128^3: 94 -> 44 us.
+static __global__ void __launch_bounds__(256, 2)
+    k_outer_pass2_pairs(Geo g, const double *__restrict__ x, const double *__restrict__ R, const double *__restrict__ src,
+                        Scalars *s, float *__restrict__ f, float *__restrict__ ab, double *__restrict__ partial)
+{
+    const size_t N = (size_t)g.n[0] * g.n[1] * g.n[2];
+    const double K2 = s->K2, nk = -K2 / 12.0;
+    const float k512 = (float)(5.0 / 12.0 * K2);
+    const double m[3] = {s->msrc[0], s->msrc[1], s->msrc[2]};
+    const bool shift = m[0] != 0.0 || m[1] != 0.0 || m[2] != 0.0;
+    float mxf[4] = {0, 0, 0, 0};
+    const unsigned nxh = (unsigned)g.n[0] >> 1, ny = (unsigned)g.n[1];
+    for (size_t pm = blockIdx.x * (size_t)blockDim.x + threadIdx.x; pm < N / 2; pm += (size_t)gridDim.x * blockDim.x) {
+        const unsigned row = (unsigned)pm / nxh, i = 2 * ((unsigned)pm - row * nxh), j = row % ny, k = row / ny;
+        const size_t c = (j + k) & 1;   // colour of the even-x cell
+        const size_t q[2] = {pm + (c ? N / 2 : 0), pm + (c ? 0 : N / 2)};
+        auto pair = [&](const double *a) { return reinterpret_cast<const double2 *>(a)[pm]; };
+        const double2 u2 = pair(x), r2 = pair(R), w02 = pair(R + N), w12 = pair(R + 2 * N), w22 = pair(R + 3 * N),
+                      aa2 = pair(R + 4 * N), rho02 = pair(src), rho22 = pair(src + N);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            auto of = [&](const double2 &v) { return h == 0 ? v.x : v.y; };
+            const double psi = psi_bg(g, (int)i + h, (int)j, (int)k, 2 * pm + h) + of(u2);
+            const double p2 = psi * psi, p4 = p2 * p2, p5 = p4 * psi;
+            const double Fp = fma(nk, p5, of(r2));
+            double F0 = of(w02), F1 = of(w12), F2 = of(w22);
+            if (shift) {
+                F0 += m[0];
+                F1 += m[1];
+                F2 += m[2];
+            }
+            const float ps = to_f32(psi), ip = 1.0f / ps, ip2 = ip * ip, ip5 = ip2 * ip2 * ip, ip6 = ip5 * ip;
+            const float fp = to_f32(Fp), w0 = to_f32(F0), w1 = to_f32(F1), w2 = to_f32(F2);
+            mxf[0] = fmaxf(mxf[0], absnanf(-8.0f * ip5 * fp));
+            mxf[1] = fmaxf(mxf[1], absnanf(ip6 * w0));
+            mxf[2] = fmaxf(mxf[2], absnanf(ip6 * w1));
+            mxf[3] = fmaxf(mxf[3], absnanf(ip6 * w2));
+            // c = dF_psi/du = -(7/8) psi^-8 AtAt + 2 pi (5 rho0 psi^4 + rho2) - (5/12) K^2 psi^4
+            const float ps2 = ps * ps, ps4 = ps2 * ps2, ip4 = ip2 * ip2;
+            const float cc = -0.875f * (ip4 * ip4) * to_f32(of(aa2)) +
+                             (float)(2.0 * kPi) * (5.0f * to_f32(of(rho02)) * ps4 + to_f32(of(rho22))) - k512 * ps4;
+            f[q[h]] = -ip5 * fp;
+            f[N + q[h]] = -w0;
+            f[2 * N + q[h]] = -w1;
+            f[3 * N + q[h]] = -w2;
+            ab[q[h]] = ip5;
+            ab[N + q[h]] = ip5 * cc;
+        }
+    }
+    __shared__ unsigned mb[4];   // block maxima, FP32 bit patterns (values >= 0)
+    if (threadIdx.x < 4) mb[threadIdx.x] = 0;
+    __syncthreads();
+#pragma unroll
+    for (int a = 0; a < 4; ++a) {
+        const unsigned v = __reduce_max_sync(0xffffffffu, __float_as_uint(mxf[a]));
+        if ((threadIdx.x & 31) == 0) atomicMax(&mb[a], v);
+    }
+    __syncthreads();
+    if (threadIdx.x < 4) partial[blockIdx.x * 4 + threadIdx.x] = (double)__uint_as_float(mb[threadIdx.x]);
+    finalize_last<4, true>(partial, gridDim.x, s->norms, &s->ticket[1]);
+}
 
 template <typename T>
 __global__ void __launch_bounds__(256) k_outer_pass2(Geo g, const double *__restrict__ x, const double *__restrict__ R,
                                                      const double *__restrict__ src, Scalars *s,
                                                      T *__restrict__ f, T *__restrict__ ab, double *__restrict__ HM,
-                                                     double *__restrict__ partial, int split, int fuse)
+                                                     double *__restrict__ partial, int split)
 {
     const size_t N = (size_t)g.n[0] * g.n[1] * g.n[2];
-    const double K2 = s->K2;
+    const double K2 = s->K2, nk = -K2 / 12.0;
     const double m0 = s->msrc[0], m1 = s->msrc[1], m2 = s->msrc[2];
-    double mx[4] = {0, 0, 0, 0};
-    float mxf[4] = {0, 0, 0, 0};
-    const bool fast = sizeof(T) == 4 && HM == nullptr;
+    unsigned long long mxu[4] = {0, 0, 0, 0};
     for (size_t p = blockIdx.x * (size_t)blockDim.x + threadIdx.x; p < N; p += (size_t)gridDim.x * blockDim.x) {
         const unsigned pu = (unsigned)p, nx = (unsigned)g.n[0], ny = (unsigned)g.n[1];
         const int i = (int)(pu % nx);
@@ -1235,36 +1438,15 @@ __global__ void __launch_bounds__(256) k_outer_pass2(Geo g, const double *__rest
         const int k = (int)(rest / ny);
         const double psi = psi_bg(g, i, j, k, p) + x[p];
         const double p2 = psi * psi, p4 = p2 * p2, p5 = p4 * psi;
-        const double Fp = fma(-K2 / 12.0, p5, R[p]);
+        const double Fp = fma(nk, p5, R[p]);
         const double Fw0 = R[N + p] + m0, Fw1 = R[2 * N + p] + m1, Fw2 = R[3 * N + p] + m2;
-        if (fast) {
-            const float ps = (float)psi, ip = 1.0f / ps, ip2 = ip * ip, ip5 = ip2 * ip2 * ip, ip6 = ip5 * ip;
-            const float fp = (float)Fp, w0 = (float)Fw0, w1 = (float)Fw1, w2 = (float)Fw2;
-            mxf[0] = fmaxf(mxf[0], absnanf(-8.0f * ip5 * fp));
-            mxf[1] = fmaxf(mxf[1], absnanf(ip6 * w0));
-            mxf[2] = fmaxf(mxf[2], absnanf(ip6 * w1));
-            mxf[3] = fmaxf(mxf[3], absnanf(ip6 * w2));
-            const size_t q = split ? (((i + j + k) & 1) ? N / 2 : 0) + (p >> 1) : p;
-            // c = dF_psi/du = -(7/8) psi^-8 AtAt + 2 pi (5 rho0 psi^4 + rho2) - (5/12) K^2 psi^4
-            const float ps2 = ps * ps, ps4 = ps2 * ps2, ip4 = ip2 * ip2;
-            const float c = -0.875f * (ip4 * ip4) * (float)R[4 * N + p] +
-                            (float)(2.0 * kPi) * (5.0f * (float)src[p] * ps4 + (float)src[N + p]) -
-                            (float)(5.0 / 12.0 * K2) * ps4;
-            f[q] = (T)(-ip5 * fp);
-            f[N + q] = (T)(-w0);
-            f[2 * N + q] = (T)(-w1);
-            f[3 * N + q] = (T)(-w2);
-            ab[q] = (T)ip5;
-            ab[N + q] = (T)(ip5 * c);
-            continue;
-        }
-        const double ip = 1.0 / psi, ip2 = ip * ip, ip5 = ip2 * ip2 * ip, ip6 = ip5 * ip;
+        const double ip = recip_f64(psi), ip2 = ip * ip, ip5 = ip2 * ip2 * ip, ip6 = ip5 * ip;
         const double H = -8.0 * ip5 * Fp;
         const double M0 = ip6 * Fw0, M1 = ip6 * Fw1, M2 = ip6 * Fw2;
-        mx[0] = fmax(mx[0], absnan(H));
-        mx[1] = fmax(mx[1], absnan(M0));
-        mx[2] = fmax(mx[2], absnan(M1));
-        mx[3] = fmax(mx[3], absnan(M2));
+        max_abs(mxu[0], H);
+        max_abs(mxu[1], M0);
+        max_abs(mxu[2], M1);
+        max_abs(mxu[3], M2);
         if (HM) {
             HM[p] = H;
             HM[N + p] = M0;
@@ -1283,13 +1465,13 @@ __global__ void __launch_bounds__(256) k_outer_pass2(Geo g, const double *__rest
             ab[N + q] = (T)(ip5 * c);
         }
     }
-    if (fast)
-        for (int a = 0; a < 4; ++a) mx[a] = (double)mxf[a];
-    double r[4];
+    double mx[4], r[4];
+#pragma unroll
+    for (int a = 0; a < 4; ++a) mx[a] = max_value(mxu[a]);
     block_max<4>(mx, r);
     if (threadIdx.x == 0)
         for (int a = 0; a < 4; ++a) partial[blockIdx.x * 4 + a] = r[a];
-    if (fuse) finalize_last<4, true>(partial, gridDim.x, s->norms, &s->ticket[1]);
+    finalize_last<4, true>(partial, gridDim.x, s->norms, &s->ticket[1]);
 }
 
 // ---------------------------------------------------------------------------------------

@@ -50,8 +50,8 @@ __global__ void __launch_bounds__(256) k_noalloc_norms(Geo g, const double *__re
                                                        double *__restrict__ partial)
 {
     const size_t N = (size_t)g.n[0] * g.n[1] * g.n[2];
-    const double K2 = s->K2;
-    double mx[4] = {0, 0, 0, 0};
+    const double nk = -s->K2 / 12.0, m[3] = {s->msrc[0], s->msrc[1], s->msrc[2]};
+    unsigned long long mxu[4] = {0, 0, 0, 0};
     for (size_t p = blockIdx.x * (size_t)blockDim.x + threadIdx.x; p < N; p += (size_t)gridDim.x * blockDim.x) {
         int i = (int)(p % g.n[0]);
         size_t rest = p / g.n[0];
@@ -59,12 +59,14 @@ __global__ void __launch_bounds__(256) k_noalloc_norms(Geo g, const double *__re
         int k = (int)(rest / g.n[1]);
         double psi = psi_background(g, i, j, k) + u[p];
         double p2 = psi * psi, p4 = p2 * p2, p5 = p4 * psi;
-        double ip = 1.0 / psi, ip2 = ip * ip, ip5 = ip2 * ip2 * ip, ip6 = ip5 * ip;
-        mx[0] = fmax(mx[0], absnan(-8.0 * ip5 * (R[p] - (K2 / 12.0) * p5)));
+        double ip = recip_f64(psi), ip2 = ip * ip, ip5 = ip2 * ip2 * ip, ip6 = ip5 * ip;
+        max_abs(mxu[0], -8.0 * ip5 * fma(nk, p5, R[p]));
 #pragma unroll
-        for (int a = 0; a < 3; ++a) mx[1 + a] = fmax(mx[1 + a], absnan(ip6 * (R[(1 + a) * N + p] + s->msrc[a])));
+        for (int a = 0; a < 3; ++a) max_abs(mxu[1 + a], ip6 * (R[(1 + a) * N + p] + m[a]));
     }
-    double r[4];
+    double mx[4], r[4];
+#pragma unroll
+    for (int a = 0; a < 4; ++a) mx[a] = max_value(mxu[a]);
     block_max<4>(mx, r);
     if (threadIdx.x == 0)
         for (int a = 0; a < 4; ++a) partial[blockIdx.x * 4 + a] = r[a];

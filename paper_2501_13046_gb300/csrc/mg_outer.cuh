@@ -163,18 +163,6 @@ __device__ __forceinline__ long long to_fixed(double x, int E)
     return (int)hi < 0 ? -v : v;
 }
 
-// 1/x to FP64 rounding: the hardware's approximate reciprocal y and one third-order step
-// y + y (r + r^2), r = 1 - x y (the geometric series of 1/(1 - r)), without the branches of the
-// IEEE division; where x y is not near 1 (x = 0, infinite or next to overflow) y is the limit itself.
-__device__ __forceinline__ double outer_recip(double x)
-{
-    double y;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    const double r = fma(-x, y, 1.0);
-    const double t = fma(y, fma(r, r, r), y);
-    return ((__double2hiint(r) >> 20) & 0x7ff) < 1023 - 10 ? t : y;   // |r| < 2^-10, not NaN
-}
-
 __device__ __forceinline__ double pow2_biased(int e) { return __hiloint2double(e << 20, 0); }   // 2^(e - 1023)
 
 // ---------------------------------------------------------------- out-of-line parts
@@ -228,7 +216,7 @@ __device__ __forceinline__ double outer_nonlin(const OuterSrc &c, double aa, dou
     const double p6 = p5 * psi, s8 = (8.0 * kPi) * p6;
 #pragma unroll
     for (int a = 0; a < 3; ++a) s[a] = s8 * c.S[a];
-    return fma(2.0 * kPi, fma(c.rho0, p5, c.rho2 * psi), (0.125 * aa) * outer_recip(p6 * psi));
+    return fma(2.0 * kPi, fma(c.rho0, p5, c.rho2 * psi), (0.125 * aa) * recip_f64(p6 * psi));
 }
 
 // ---------------------------------------------------------------- the fused residual
