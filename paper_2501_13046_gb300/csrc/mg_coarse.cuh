@@ -176,6 +176,123 @@ __global__ void __launch_bounds__(1024) k_gauss_jordan(C *__restrict__ gaug, int
     }
 }
 
+// Inverse of a matrix of order m <= 32 R held in registers: lane i0 of warp j0 holds the entries (i0 + 32 a,
+// j0 + 8 b), so one column lives in one warp.  In-place Gauss-Jordan with partial pivoting and no row
+// exchanges: step k takes the largest entry of column k among the rows not used yet (first of equals), row p_k
+// plays row k from then on, and the inverse's entry (k, p_j) ends in place (p_k, j).  Per step the
+// column's warp finds the pivot with two warp reductions and publishes the column in shared memory (double
+// buffered); after one barrier every warp takes the pivot row's entries of its own columns by shuffles and
+// eliminates, the next column's warp that column first.  Reads the left block of the assembled
+// [A | I] (row stride 2m).  A zero or NaN pivot yields non-finite entries, as in k_gauss_jordan (which
+// the W block, of order up to 400, takes once per context).
+template <typename T, int R>
+__global__ void __launch_bounds__(256) k_invert_registers(const T *__restrict__ aug, int m, T *__restrict__ inv)
+{
+    constexpr int NC = 4 * R;
+    __shared__ T col[2][32 * R];
+    __shared__ T ip_s[2];
+    __shared__ int piv_s[32 * R], step_s[32 * R];   // row of step k; step of row i
+    const int i0 = threadIdx.x & 31, j0 = threadIdx.x >> 5;
+    T A[R][NC];
+    unsigned used = 0;   // bit a: row i0 + 32 a has been a pivot row
+#pragma unroll
+    for (int a = 0; a < R; ++a)
+#pragma unroll
+        for (int b = 0; b < NC; ++b) {
+            const int i = i0 + 32 * a, j = j0 + 8 * b;
+            A[a][b] = (i < m && j < m) ? aug[(size_t)i * 2 * m + j] : (T)0;
+        }
+    // column k's warp (c: the column's entries): its pivot, and the column as the elimination factors of step k
+    auto publish = [&](int k, const T (&c)[R]) {
+        const int buf = k & 1;
+        // compared as bit patterns (FP32: exact; FP64: the high word decides, which is enough to choose a pivot)
+        unsigned best = 0, row = 0xffffffffu;
+#pragma unroll
+        for (int a = 0; a < R; ++a) {
+            unsigned v;
+            if constexpr (sizeof(T) == 4) v = __float_as_uint(c[a]) & 0x7fffffffu;
+            else v = (unsigned)__double2hiint(c[a]) & 0x7fffffffu;
+            if (i0 + 32 * a < m && !((used >> a) & 1) && (row == 0xffffffffu || v > best)) {
+                best = v;
+                row = i0 + 32 * a;
+            }
+        }
+        const unsigned top = __reduce_max_sync(0xffffffffu, row == 0xffffffffu ? 0u : best);
+        const unsigned p = __reduce_min_sync(0xffffffffu, row != 0xffffffffu && best == top ? row : 0xffffffffu);
+#pragma unroll
+        for (int a = 0; a < R; ++a) {
+            col[buf][i0 + 32 * a] = c[a];
+            if (i0 + 32 * a == (int)p) {
+                ip_s[buf] = (T)1 / c[a];
+                piv_s[k] = (int)p;
+                step_s[p] = k;
+            }
+        }
+    };
+    if (j0 == 0) {
+        T c[R];
+#pragma unroll
+        for (int a = 0; a < R; ++a) c[a] = A[a][0];
+        publish(0, c);
+    }
+    __syncthreads();
+    for (int k = 0; k < m; ++k) {
+        const T ip = ip_s[k & 1];
+        const int p = piv_s[k], pa = p >> 5;
+        T f[R];
+        bool is_p[R];
+#pragma unroll
+        for (int a = 0; a < R; ++a) {
+            f[a] = col[k & 1][i0 + 32 * a];
+            is_p[a] = i0 + 32 * a == p;
+            used |= is_p[a] ? 1u << a : 0u;
+        }
+        // one column: c - f (pivot row's entry / pivot), the pivot row itself scaled
+        auto eliminated = [&](const T (&c)[R], T (&o)[R]) {
+            T vp = c[0];
+#pragma unroll
+            for (int a = 1; a < R; ++a) vp = a == pa ? c[a] : vp;
+            const T pr = __shfl_sync(0xffffffffu, vp, p & 31) * ip;
+#pragma unroll
+            for (int a = 0; a < R; ++a) o[a] = is_p[a] ? pr : c[a] - f[a] * pr;
+        };
+        // the next column first, on a copy, so that its pivot search overlaps the elimination below
+        if (k + 1 < m && j0 == ((k + 1) & 7)) {
+            const int nb = (k + 1) >> 3;
+            T c[R], o[R];
+#pragma unroll
+            for (int a = 0; a < R; ++a) {
+                c[a] = A[a][0];
+#pragma unroll
+                for (int b = 1; b < NC; ++b) c[a] = b == nb ? A[a][b] : c[a];
+            }
+            eliminated(c, o);
+            publish(k + 1, o);
+        }
+        // every column (no branches inside: the columns' shuffles overlap); column k becomes the inverse's
+#pragma unroll
+        for (int b = 0; b < NC; ++b) {
+            if (8 * b >= m) break;
+            T c[R], o[R];
+#pragma unroll
+            for (int a = 0; a < R; ++a) c[a] = A[a][b];
+            eliminated(c, o);
+            const bool diag = j0 + 8 * b == k;
+#pragma unroll
+            for (int a = 0; a < R; ++a) A[a][b] = diag ? (is_p[a] ? ip : -f[a] * ip) : o[a];
+        }
+        __syncthreads();
+    }
+#pragma unroll
+    for (int a = 0; a < R; ++a)
+        if (i0 + 32 * a < m) {
+            const int r = step_s[i0 + 32 * a];
+#pragma unroll
+            for (int b = 0; b < NC; ++b)
+                if (j0 + 8 * b < m) inv[(size_t)r * m + piv_s[j0 + 8 * b]] = A[a][b];
+        }
+}
+
 // Coarsest-level correction: e_psi = Gpsi[0:N, 0:N] f_psi, e_W = GW[0:3N, 0:3N] f_W (the
 // bordered rows and columns belong to the multipliers; their right-hand side is zero).  One
 // warp per output row; FP32 rows accumulate in FP32, FP64 rows in FP64.

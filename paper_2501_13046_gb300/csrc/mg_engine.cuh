@@ -272,7 +272,7 @@ inline size_t gj_smem(int m)
 }
 
 // Inverse of the coarsest psi row for this outer iteration (its coefficients were just restricted),
-// on a parallel branch: the one-CTA elimination overlaps the first cycle's descent, and the first
+// on a parallel branch: the one-CTA inversion overlaps the first cycle's descent, and the first
 // coarse solve of the iteration waits for it (enqueue_coarse).
 template <typename T, int ORDER, int BC>
 mg_status enqueue_dense_psi_inverse(mg_ctx *x)
@@ -280,14 +280,19 @@ mg_status enqueue_dense_psi_inverse(mg_ctx *x)
     LevelBufs &C = x->lev[x->nlev - 1];
     const int periodic = x->cfg.bc == MG_BC_PERIODIC;
     Coef<T> cf = make_coef<T>(C.geo, x->cfg.order);
-    const size_t sm = gj_smem<T>(x->mpsi);
     CK(cudaEventRecord(x->ev_fork, x->stream));
     CK(cudaStreamWaitEvent(x->side, x->ev_fork, 0));
     with_bc<BC>([&](auto B) {
         k_dense_psi_assemble<T, T, ORDER, decltype(B)::value><<<1, 512, 0, x->side>>>(C.geo, cf, (const T *)C.c,
                                                                                     (T *)x->gj, periodic);
     });
-    k_gauss_jordan<T, T><<<1, 1024, sm, x->side>>>((T *)x->gj, x->mpsi, sm > 0, (T *)x->Gpsi);
+    const int m = x->mpsi;   // at most (kDenseMaxW - 3) / 3 + 1 = 133
+    const T *gj = (const T *)x->gj;
+    T *G = (T *)x->Gpsi;
+    if (m <= 32) k_invert_registers<T, 1><<<1, 256, 0, x->side>>>(gj, m, G);
+    else if (m <= 64) k_invert_registers<T, 2><<<1, 256, 0, x->side>>>(gj, m, G);
+    else if (m <= 96) k_invert_registers<T, 3><<<1, 256, 0, x->side>>>(gj, m, G);
+    else k_invert_registers<T, 5><<<1, 256, 0, x->side>>>(gj, m, G);
     CK(cudaGetLastError());
     CK(cudaEventRecord(x->ev_join, x->side));
     x->join_pending = true;
@@ -373,9 +378,7 @@ mg_status engine_prepare(mg_ctx *x)
         if (cudaFuncSetAttribute(k_coarse_cycle<T, ORDER, decltype(B)::value>,
                                  cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxCoarseSmem) != cudaSuccess)
             st = fail(MG_ERR_CUDA, "cudaFuncSetAttribute(k_coarse_cycle)");
-        if (cudaFuncSetAttribute(k_gauss_jordan<T, T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)kMaxCoarseSmem) != cudaSuccess ||
-            cudaFuncSetAttribute(k_gauss_jordan<double, T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        if (cudaFuncSetAttribute(k_gauss_jordan<double, T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)kMaxCoarseSmem) != cudaSuccess)
             st = fail(MG_ERR_CUDA, "cudaFuncSetAttribute(k_gauss_jordan)");
         if (cudaFuncSetAttribute(k_smooth_tile<T, ORDER, BC, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize,
