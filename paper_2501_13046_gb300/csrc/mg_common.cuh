@@ -16,6 +16,7 @@
 #include "mg_tile.cuh"
 #include "mg_outer.cuh"
 #include "mg_coarse.cuh"
+#include "mg_cluster.cuh"
 
 namespace ctt {
 
@@ -205,6 +206,7 @@ struct mg_ctx {
     double *R = nullptr;     // 5N: outer pass-1 output
     int dense = 0;           // 1: the coarsest level is solved with the dense inverses below
     int fused = 0;           // 1: the next-to-coarsest level's cycle runs in one CTA (k_coarse_cycle)
+    int cluster = -1;        // >= 0: the cycle from this level down runs in one cluster (k_cluster_cycle)
     int mpsi = 0, mw = 0;    // orders of the (bordered) psi and W systems
     void *Gpsi = nullptr;    // mpsi^2 T: inverse of the psi row (per outer iteration)
     void *GW = nullptr;      // mw^2 T: inverse of the W rows (once, at creation)

@@ -163,6 +163,52 @@ mg_status enqueue_coarse(mg_ctx *x, int l)
 // the residual is restricted once; the coarser level is then cycled gamma times on that right-
 // hand side (1: V-cycle, 2: W-cycle), the later visits continuing from its correction, and the
 // result is prolongated and post-smoothed.  The coarsest level is visited once (exact solve).
+// The cycle of level l and every level below it in one cluster launch.
+template <typename T, int ORDER, int BC>
+mg_status enqueue_cluster(mg_ctx *x, int l, bool zero)
+{
+    const int Lc = x->nlev - 1;
+    LevelBufs &L = x->lev[l];
+    if (zero) L.curB = 0;
+    if (x->join_pending) {
+        CK(cudaStreamWaitEvent(x->stream, x->ev_join, 0));
+        x->join_pending = false;
+    }
+    ClusterArgs<T> a;
+    std::memset(&a, 0, sizeof(a));
+    Geo geo[kClusterLevels];
+    a.nl = Lc - l;
+    for (int k = 0; k < a.nl; ++k) {
+        geo[k] = x->lev[l + k].geo;
+        a.lev[k] = ClusterLevel<T>{geo[k], make_coef<T>(geo[k], x->cfg.order, x->omega), (const T *)x->lev[l + k].c};
+    }
+    a.gc = x->lev[Lc].geo;
+    a.zero = zero;
+    a.nu_pre = x->cfg.nu_pre;
+    a.nu_post = x->cfg.nu_post;
+    a.f = (const T *)L.f;
+    a.e_in = zero ? (const T *)L.eA : (const T *)L.cur();
+    a.e_out = (T *)L.alt();
+    a.Gpsi = (const T *)x->Gpsi;
+    a.GW = (const T *)x->GW;
+    a.mpsi = x->mpsi;
+    a.mw = x->mw;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(kClusterCtas);
+    cfg.blockDim = dim3(kClusterThreads);
+    cfg.dynamicSmemBytes = cluster_smem_bytes(geo, a.nl, a.gc, x->cfg.bc == MG_BC_ROBIN, sizeof(T));
+    cfg.stream = x->stream;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = kClusterCtas;
+    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    CK(cudaLaunchKernelEx(&cfg, k_cluster_cycle<T, ORDER, BC>, a));
+    L.curB ^= 1;
+    return MG_OK;
+}
+
 template <typename T, int ORDER, int BC>
 mg_status enqueue_cycle(mg_ctx *x, int l, bool zero)
 {
@@ -177,6 +223,7 @@ mg_status enqueue_cycle(mg_ctx *x, int l, bool zero)
         if (x->join_pending) {
             CK(cudaStreamWaitEvent(x->stream, x->ev_join, 0));
             x->join_pending = false;
+    if (l == x->cluster) return enqueue_cluster<T, ORDER, BC>(x, l, zero);   // this level and all below in one cluster
         }
         const T *ein = zero ? (const T *)L.eA : (const T *)L.cur();
         size_t smem =
@@ -398,6 +445,9 @@ mg_status engine_prepare(mg_ctx *x)
 // Back-to-back launches of one kernel between events (measurement aid).
 template <typename T, int ORDER, int BC>
 mg_status engine_time_kernel(mg_ctx *x, int which, int reps, float *ms)
+        if (cudaFuncSetAttribute(k_cluster_cycle<T, ORDER, BC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)kMaxCoarseSmem) != cudaSuccess)
+            st = fail(MG_ERR_CUDA, "cudaFuncSetAttribute(k_cluster_cycle)");
 {
     LevelBufs &L = x->lev[0];
     Coef<T> cf = make_coef<T>(L.geo, x->cfg.order);
