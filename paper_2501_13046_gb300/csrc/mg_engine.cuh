@@ -30,8 +30,8 @@ inline Regions restrict_regions(const Geo &gc, int *grid, int threads)
     long long ix = gc.n[0] - 2, iy = gc.n[1] - 2, iz = gc.n[2] - 2;
     size_t nint = (ix > 0 && iy > 0 && iz > 0) ? (size_t)ix * iy * iz : 0;
     size_t nsh = shell_count(gc.n, 1);
-    int bi = nint ? grid_for(nint, 1 << 24, threads) : 0;
-    int bs = nsh ? grid_for(nsh, 152 * 4, threads) : 0;
+    int bi = nint ? grid_for(8 * nint, 1 << 24, threads) : 0;   // 8 threads per coarse cell
+    int bs = nsh ? grid_for(8 * nsh, 152 * 8, threads) : 0;
     r.nblk_sh = bs;
     *grid = std::max(1, bi + bs);
     return r;
@@ -90,9 +90,10 @@ mg_status enqueue_restrict(mg_ctx *x, int l)
 }
 
 // `sweeps` red-black sweeps on a colour-split level.  Each sweep reads the current buffer and
-// writes the alternate one (red half, then black half), then the two swap roles.
+// writes the alternate one (red half, then black half), then the two swap roles.  zero: the correction
+// is zero (its buffer need not hold zeros; sweeps >= 1).
 template <typename T, int ORDER, int BC>
-mg_status enqueue_sweeps(mg_ctx *x, int l, int sweeps)
+mg_status enqueue_sweeps(mg_ctx *x, int l, int sweeps, bool zero = false)
 {
     LevelBufs &L = x->lev[l];
     Coef<T> cf = make_coef<T>(L.geo, x->cfg.order, x->omega);
@@ -104,7 +105,11 @@ mg_status enqueue_sweeps(mg_ctx *x, int l, int sweeps)
         T *Y = (T *)L.alt();
         for (int colour = 0; colour < 2; ++colour) {
             const T *O = colour == 0 ? X : Y;
-            if (L.tiled) {
+            if (zero && s == 0 && colour == 0) {
+                k_smooth_first<T, BC><<<grid_for(L.N / 2, 152 * 8), kThreads, 0, x->stream>>>(
+                    L.geo, cf.fd, cf.dl, cf.idW[0], cf.idW[1], cf.idW[2], cf.iom, (T *)L.cur(), Y, (const T *)L.f,
+                    (const T *)L.c);
+            } else if (L.tiled) {
                 const CUtensorMap &mO = colour == 0 ? L.tm_cur() : L.tm_alt();
                 CKS(launch_tile<T, ORDER, BC>(x, L, tc, L.tm_cur(), mO, X, O, Y, colour));
             } else {
@@ -158,11 +163,6 @@ mg_status enqueue_coarse(mg_ctx *x, int l)
     return fail(MG_ERR_UNSUPPORTED, "coarsest level too large for the one-CTA coarse solve; use more levels");
 }
 
-// One multigrid cycle on J e = f at level l (the coarsest level is solved directly).  zero: the
-// level's correction starts at zero, else the cycle continues from it.  After pre-smoothing
-// the residual is restricted once; the coarser level is then cycled gamma times on that right-
-// hand side (1: V-cycle, 2: W-cycle), the later visits continuing from its correction, and the
-// result is prolongated and post-smoothed.  The coarsest level is visited once (exact solve).
 // The cycle of level l and every level below it in one cluster launch.
 template <typename T, int ORDER, int BC>
 mg_status enqueue_cluster(mg_ctx *x, int l, bool zero)
@@ -209,6 +209,11 @@ mg_status enqueue_cluster(mg_ctx *x, int l, bool zero)
     return MG_OK;
 }
 
+// One multigrid cycle on J e = f at level l (the coarsest level is solved directly).  zero: the
+// level's correction starts at zero, else the cycle continues from it.  After pre-smoothing
+// the residual is restricted once; the coarser level is then cycled gamma times on that right-
+// hand side (1: V-cycle, 2: W-cycle), the later visits continuing from its correction, and the
+// result is prolongated and post-smoothed.  The coarsest level is visited once (exact solve).
 template <typename T, int ORDER, int BC>
 mg_status enqueue_cycle(mg_ctx *x, int l, bool zero)
 {
@@ -218,12 +223,12 @@ mg_status enqueue_cycle(mg_ctx *x, int l, bool zero)
         L.curB = 0;
         return enqueue_coarse<T, ORDER, BC>(x, Lc);
     }
+    if (l == x->cluster) return enqueue_cluster<T, ORDER, BC>(x, l, zero);   // this level and all below in one cluster
     if (x->fused && l == Lc - 1) {   // this level and the coarsest in one CTA
         LevelBufs &C = x->lev[Lc];
         if (x->join_pending) {
             CK(cudaStreamWaitEvent(x->stream, x->ev_join, 0));
             x->join_pending = false;
-    if (l == x->cluster) return enqueue_cluster<T, ORDER, BC>(x, l, zero);   // this level and all below in one cluster
         }
         const T *ein = zero ? (const T *)L.eA : (const T *)L.cur();
         size_t smem =
@@ -243,17 +248,19 @@ mg_status enqueue_cycle(mg_ctx *x, int l, bool zero)
     }
     if (zero) {
         L.curB = 0;
-        CK(cudaMemsetAsync(L.eA, 0, 4 * L.N * sizeof(T), x->stream));
+        if (x->cfg.nu_pre == 0) CK(cudaMemsetAsync(L.eA, 0, 4 * L.N * sizeof(T), x->stream));
     }
-    CKS(enqueue_sweeps<T, ORDER, BC>(x, l, x->cfg.nu_pre));
+    CKS(enqueue_sweeps<T, ORDER, BC>(x, l, x->cfg.nu_pre, zero));
     LevelBufs &C = x->lev[l + 1];
     CKS(enqueue_restrict<T, ORDER, BC>(x, l));
     const int visits = l + 1 == Lc ? 1 : x->gamma;
     for (int v = 0; v < visits; ++v) CKS(enqueue_cycle<T, ORDER, BC>(x, l + 1, v == 0));
-    with_bc<BC>([&](auto B) {
-        k_prolong_add<T, decltype(B)::value><<<grid_for(L.N, 1 << 24, x->threads), x->threads, 0, x->stream>>>(
+    if constexpr (BC == BC_SYM)   // mirrored and extrapolated parents
+        k_prolong_add<T, BC><<<grid_for(L.N, 1 << 24, x->threads), x->threads, 0, x->stream>>>(
             L.geo, C.geo, (const T *)C.cur(), (T *)L.cur(), C.split);
-    });
+    else
+        k_prolong_blocks<T, BC><<<dim3(grid_for(C.N, 1 << 24, 128), 4), 128, 0, x->stream>>>(L.geo, C.geo, (const T *)C.cur(),
+                                                                                   (T *)L.cur(), C.split);
     CK(cudaGetLastError());
     return enqueue_sweeps<T, ORDER, BC>(x, l, x->cfg.nu_post);
 }
@@ -438,6 +445,9 @@ mg_status engine_prepare(mg_ctx *x)
         if (cudaFuncSetAttribute(k_outer_residual<ORDER, BC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)outer_smem_bytes<ORDER>()) != cudaSuccess)
             st = fail(MG_ERR_CUDA, "cudaFuncSetAttribute(k_outer_residual)");
+        if (cudaFuncSetAttribute(k_cluster_cycle<T, ORDER, BC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)kMaxCoarseSmem) != cudaSuccess)
+            st = fail(MG_ERR_CUDA, "cudaFuncSetAttribute(k_cluster_cycle)");
     });
     return st;
 }
@@ -445,9 +455,6 @@ mg_status engine_prepare(mg_ctx *x)
 // Back-to-back launches of one kernel between events (measurement aid).
 template <typename T, int ORDER, int BC>
 mg_status engine_time_kernel(mg_ctx *x, int which, int reps, float *ms)
-        if (cudaFuncSetAttribute(k_cluster_cycle<T, ORDER, BC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)kMaxCoarseSmem) != cudaSuccess)
-            st = fail(MG_ERR_CUDA, "cudaFuncSetAttribute(k_cluster_cycle)");
 {
     LevelBufs &L = x->lev[0];
     Coef<T> cf = make_coef<T>(L.geo, x->cfg.order);

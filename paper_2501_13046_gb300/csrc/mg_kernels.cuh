@@ -764,35 +764,57 @@ __global__ void __launch_bounds__(256, 2) k_smooth_colour(Geo g, Coef<T> cf, con
     }
 }
 
+// The first colour pass (colour 0) of a correction that starts at zero: J e = 0, so the new values need no
+// stencil and no old values.  Also clears X's colour-1 half, which the next pass reads as its old
+// values (so no clearing pass is needed).  Same values as the general pass on zeros.  128^3: 10 us for the 33 us
+// of the tiled pass and the 7 us of the clearing.
+template <typename T, int BC>
+__global__ void __launch_bounds__(256) k_smooth_first(Geo g, FaceDiag<T> fd, T dl0, T idW0, T idW1, T idW2, T iom,
+                                                      T *__restrict__ X, T *__restrict__ Y, const T *__restrict__ f,
+                                                      const T *__restrict__ ab)
+{
+    const unsigned nxh = (unsigned)g.n[0] >> 1, ny = (unsigned)g.n[1], Nh = nxh * ny * (unsigned)g.n[2];
+    const size_t N = 2 * (size_t)Nh;
+    const T idW[3] = {idW0, idW1, idW2};
+    for (unsigned m = blockIdx.x * blockDim.x + threadIdx.x; m < Nh; m += gridDim.x * blockDim.x) {
+        const unsigned row = m / nxh, j = row % ny, k = row / ny;
+        const T ca = ab[m], cb = ab[N + m];
+        T fv[4];
+#pragma unroll
+        for (int a = 0; a < 4; ++a) fv[a] = f[a * N + m];
+        T dl, kW[3];
+        relax_factors<BC>(fd, g, (int)(2 * (m - row * nxh) + ((j + k) & 1)), (int)j, (int)k, true, dl0, idW, iom, dl, kW);
+        Y[m] = fv[0] / ((ca * dl + cb) * iom);
+#pragma unroll
+        for (int a = 0; a < 3; ++a) Y[(1 + a) * N + m] = fv[1 + a] * kW[a];
+#pragma unroll
+        for (int a = 0; a < 4; ++a) X[a * N + Nh + m] = 0;
+    }
+}
+
 // Residual r = f - J e on a colour-split fine level, averaged over the 8 children into the
 // coarse rhs (stored colour-split, or plain when the coarse level is the coarsest).  Blocks
 // [0, nblk_sh) take the coarse shell, the others the coarse cells whose children's stencils stay
 // inside the fine box (the coarse interior box [1, nc-1)^3).
+// One thread per child, the 8 children of a coarse cell in 8 neighbouring lanes (their sum by shuffles):
+// with one thread per coarse cell the 8 stencils ran one after the other on an eighth of the threads (64^3 FP64: 143 us
+// per launch, 32^3: 141 us).
 template <typename T, int ORDER, int BC, bool INTERIOR>
-__device__ __forceinline__ void restrict_cell(const Geo &g, const Coef<T> &cf, const Geo &gc, const T *e, const T *f,
-                                              const T *ab, T *fc, size_t N, size_t Nc, int csplit, int I, int J, int K)
+__device__ __forceinline__ void restrict_child(const Geo &g, const Coef<T> &cf, const T *e, const T *f, const T *ab,
+                                               size_t N, int i, int j, int k, T r[4])
 {
-    T acc[4] = {0, 0, 0, 0};
-#pragma unroll 1
-    for (int d = 0; d < 8; ++d) {
-        int i = 2 * I + (d & 1), j = 2 * J + ((d >> 1) & 1), k = 2 * K + (d >> 2);
-        size_t p = sidx(g, i, j, k, N, 1);
-        T Je[4], ctr[4];
-        apply_J_split<T, ORDER, BC, INTERIOR>(e, e, N, g, i, j, k, ab[p], ab[N + p], cf, Je, ctr);
+    const size_t p = sidx(g, i, j, k, N, 1);
+    T Je[4], ctr[4];
+    apply_J_split<T, ORDER, BC, INTERIOR>(e, e, N, g, i, j, k, ab[p], ab[N + p], cf, Je, ctr);
 #pragma unroll
-        for (int a = 0; a < 4; ++a) acc[a] += f[a * N + p] - Je[a];
-    }
-    size_t pc = sidx(gc, I, J, K, Nc, csplit);
-#pragma unroll
-    for (int a = 0; a < 4; ++a) fc[a * Nc + pc] = acc[a] * (T)0.125;
+    for (int a = 0; a < 4; ++a) r[a] = f[a * N + p] - Je[a];
 }
 
 template <typename T, int ORDER, int BC>
-__device__ __noinline__ void restrict_cell_shell(const Geo &g, const Coef<T> &cf, const Geo &gc, const T *e,
-                                                 const T *f, const T *ab, T *fc, size_t N, size_t Nc, int csplit,
-                                                 int I, int J, int K)
+__device__ __noinline__ void restrict_child_shell(const Geo &g, const Coef<T> &cf, const T *e, const T *f, const T *ab,
+                                                  size_t N, int i, int j, int k, T *r)
 {
-    restrict_cell<T, ORDER, BC, false>(g, cf, gc, e, f, ab, fc, N, Nc, csplit, I, J, K);
+    restrict_child<T, ORDER, BC, false>(g, cf, e, f, ab, N, i, j, k, *reinterpret_cast<T(*)[4]>(r));
 }
 
 template <typename T, int ORDER, int BC>
@@ -802,23 +824,38 @@ __global__ void __launch_bounds__(256, 2) k_residual_restrict(Geo g, Coef<T> cf,
 {
     const size_t N = (size_t)g.n[0] * g.n[1] * g.n[2];
     const size_t Nc = (size_t)gc.n[0] * gc.n[1] * gc.n[2];
-    int I, J, K;
-    if ((int)blockIdx.x >= rg.nblk_sh) {
-        // coarse interior box [1, nc-1)^3, x fastest
-        const int ix = gc.n[0] - 2, iy = gc.n[1] - 2, iz = gc.n[2] - 2;
-        const unsigned total = (ix > 0 && iy > 0 && iz > 0) ? (unsigned)ix * iy * iz : 0;
-        const unsigned stride = (unsigned)(gridDim.x - rg.nblk_sh) * blockDim.x;
-        for (unsigned t = (blockIdx.x - rg.nblk_sh) * blockDim.x + threadIdx.x; t < total; t += stride) {
-            const unsigned r = t / (unsigned)ix;
-            I = 1 + (int)(t - r * (unsigned)ix);
-            J = 1 + (int)(r % (unsigned)iy);
-            K = 1 + (int)(r / (unsigned)iy);
-            restrict_cell<T, ORDER, BC, true>(g, cf, gc, e, f, ab, fc, N, Nc, csplit, I, J, K);
+    const bool inner = (int)blockIdx.x >= rg.nblk_sh;
+    // coarse interior box [1, nc-1)^3, x fastest, or the coarse shell
+    const int ix = gc.n[0] - 2, iy = gc.n[1] - 2, iz = gc.n[2] - 2;
+    const unsigned total = inner ? ((ix > 0 && iy > 0 && iz > 0) ? (unsigned)ix * iy * iz : 0) : (unsigned)shell_count(gc.n, 1);
+    const unsigned blk = inner ? blockIdx.x - rg.nblk_sh : blockIdx.x;
+    const unsigned stride = (inner ? gridDim.x - rg.nblk_sh : (unsigned)rg.nblk_sh) * (blockDim.x >> 3);
+    const int d = threadIdx.x & 7;
+    for (unsigned t0 = (blk * blockDim.x + (threadIdx.x & ~31u)) >> 3; t0 < total; t0 += stride) {   // a warp's 4 cells
+        const unsigned t = t0 + ((threadIdx.x & 31) >> 3);
+        int I = 0, J = 0, K = 0;
+        T r[4] = {0, 0, 0, 0};
+        if (t < total) {
+            if (inner) {
+                const unsigned q = t / (unsigned)ix;
+                I = 1 + (int)(t - q * (unsigned)ix);
+                J = 1 + (int)(q % (unsigned)iy);
+                K = 1 + (int)(q / (unsigned)iy);
+                restrict_child<T, ORDER, BC, true>(g, cf, e, f, ab, N, 2 * I + (d & 1), 2 * J + ((d >> 1) & 1),
+                                                   2 * K + (d >> 2), r);
+            } else {
+                shell_cell(gc, 1, t, I, J, K);
+                restrict_child_shell<T, ORDER, BC>(g, cf, e, f, ab, N, 2 * I + (d & 1), 2 * J + ((d >> 1) & 1),
+                                                   2 * K + (d >> 2), r);
+            }
         }
-    } else {
-        const unsigned stride = (unsigned)rg.nblk_sh * blockDim.x;
-        for (unsigned t = blockIdx.x * blockDim.x + threadIdx.x; shell_cell(gc, 1, t, I, J, K); t += stride)
-            restrict_cell_shell<T, ORDER, BC>(g, cf, gc, e, f, ab, fc, N, Nc, csplit, I, J, K);
+#pragma unroll
+        for (int a = 0; a < 4; ++a)
+            for (int o = 1; o < 8; o <<= 1) r[a] += __shfl_xor_sync(0xffffffffu, r[a], o);
+        if (t < total && d < 4) {   // lane d writes field d
+            const T v = d == 0 ? r[0] : d == 1 ? r[1] : d == 2 ? r[2] : r[3];
+            fc[d * Nc + sidx(gc, I, J, K, Nc, csplit)] = v * (T)0.125;
+        }
     }
 }
 
@@ -907,6 +944,109 @@ __global__ void __launch_bounds__(256) k_prolong_add(Geo g, Geo gc, const T *__r
 #pragma unroll
             for (int d = 0; d < 8; ++d) s = fma(bc_signed<BC>(w[d], mir[d], a), e[idx[d]], s);
             ef[(size_t)a * N + q] += s;
+        }
+    }
+}
+
+template <typename T>
+__device__ __noinline__ T robin_ratio_call(const Geo &g, int bi, int bj, int bk, int gi, int gj, int gk)
+{
+    return robin_ratio<T>(g, bi, bj, bk, gi, gj, gk);
+}
+
+// k_prolong_add for periodic and Robin boxes, one thread per coarse cell and field: its 2 x 2 x 2 fine cells share the
+// 27 coarse values around it (3.4 reads per fine cell and field instead of 8), combined axis by axis.  A thread's
+// x pairs are one cell of each colour at the same storage place, so fine accesses are contiguous over a
+// warp.  128^3: 32 us with one thread per fine cell.
+template <typename T, int BC>
+__global__ void __launch_bounds__(128) k_prolong_blocks(Geo g, Geo gc, const T *__restrict__ ec, T *__restrict__ ef,
+                                                        int csplit)
+{
+    const unsigned ncx = gc.n[0], ncy = gc.n[1], ncz = gc.n[2], Nc = ncx * ncy * ncz, nxh = ncx;   // nx / 2 = ncx
+    const size_t N = 8 * (size_t)Nc, Nh = N / 2;
+    for (unsigned c = blockIdx.x * blockDim.x + threadIdx.x; c < Nc; c += gridDim.x * blockDim.x) {
+        const unsigned r = c / ncx;
+        const int I = (int)(c - r * ncx), J = (int)(r % ncy), K = (int)(r / ncy);
+        // neighbour places per axis under the boundary rule
+        int p[3][3];
+        const int at[3] = {I, J, K};
+#pragma unroll
+        for (int a = 0; a < 3; ++a)
+#pragma unroll
+            for (int d = 0; d < 3; ++d) {
+                int q = at[a] + d - 1;
+                const int n = gc.n[a];
+                if constexpr (BC == BC_PERIODIC) q += q < 0 ? n : (q >= n ? -n : 0);
+                else q = min(max(q, 0), n - 1);
+                p[a][d] = q;
+            }
+        const bool edge = BC != BC_PERIODIC && (I == 0 || J == 0 || K == 0 || I == gc.n[0] - 1 || J == gc.n[1] - 1 || K == gc.n[2] - 1);
+        auto place = [&](int x, int y, int z) -> unsigned {   // (31-bit cell counts)
+            const unsigned lin = (unsigned)x + ncx * ((unsigned)y + ncy * (unsigned)z);
+            return csplit ? (((x + y + z) & 1) ? Nc / 2 : 0u) + (lin >> 1) : lin;
+        };
+        {
+            const int a = blockIdx.y;   // field
+            const T *e = ec + (size_t)a * Nc;
+            T *o = ef + (size_t)a * N;
+            T s[2][2][2], old[2][2][2];   // [z][y][x] fine cell of the block
+            size_t at2[2][2];             // storage place of the pair of row (y, z) in its colour halves
+#pragma unroll
+            for (int z = 0; z < 2; ++z)
+#pragma unroll
+                for (int y = 0; y < 2; ++y) {
+                    at2[z][y] = (size_t)I + (size_t)nxh * ((unsigned)(2 * J + y) + 2 * ncy * (unsigned)(2 * K + z));
+                    const bool odd = (y + z) & 1;   // colour of the pair's even-x cell ((j + k) & 1)
+                    old[z][y][0] = o[at2[z][y] + (odd ? Nh : 0)];
+                    old[z][y][1] = o[at2[z][y] + (odd ? 0 : Nh)];
+                }
+#pragma unroll
+            for (int z = 0; z < 3; ++z) {
+                T ty[2][2];   // rows of this coarse plane combined along x and y
+#pragma unroll
+                for (int y = 0; y < 3; ++y) {
+                    T v[3];
+#pragma unroll
+                    for (int x = 0; x < 3; ++x) {
+                        v[x] = e[place(p[0][x], p[1][y], p[2][z])];
+                        if (edge && (I + x - 1 != p[0][x] || J + y - 1 != p[1][y] || K + z - 1 != p[2][z]))
+                            v[x] *= robin_ratio_call<T>(gc, p[0][x], p[1][y], p[2][z], I + x - 1, J + y - 1, K + z - 1);
+                    }
+                    const T x0 = (T)0.75 * v[1] + (T)0.25 * v[0], x1 = (T)0.75 * v[1] + (T)0.25 * v[2];
+                    if (y == 0) {
+                        ty[0][0] = (T)0.25 * x0;
+                        ty[0][1] = (T)0.25 * x1;
+                    } else if (y == 1) {
+                        ty[0][0] = fma((T)0.75, x0, ty[0][0]);
+                        ty[0][1] = fma((T)0.75, x1, ty[0][1]);
+                        ty[1][0] = (T)0.75 * x0;
+                        ty[1][1] = (T)0.75 * x1;
+                    } else {
+                        ty[1][0] = fma((T)0.25, x0, ty[1][0]);
+                        ty[1][1] = fma((T)0.25, x1, ty[1][1]);
+                    }
+                }
+#pragma unroll
+                for (int y = 0; y < 2; ++y)
+#pragma unroll
+                    for (int x = 0; x < 2; ++x) {
+                        if (z == 0) s[0][y][x] = (T)0.25 * ty[y][x];
+                        else if (z == 1) {
+                            s[0][y][x] = fma((T)0.75, ty[y][x], s[0][y][x]);
+                            s[1][y][x] = (T)0.75 * ty[y][x];
+                        } else {
+                            s[1][y][x] = fma((T)0.25, ty[y][x], s[1][y][x]);
+                        }
+                    }
+            }
+#pragma unroll
+            for (int z = 0; z < 2; ++z)
+#pragma unroll
+                for (int y = 0; y < 2; ++y) {
+                    const bool odd = (y + z) & 1;
+                    o[at2[z][y] + (odd ? Nh : 0)] = old[z][y][0] + s[z][y][0];
+                    o[at2[z][y] + (odd ? 0 : Nh)] = old[z][y][1] + s[z][y][1];
+                }
         }
     }
 }
