@@ -236,20 +236,21 @@ __global__ void __launch_bounds__(128) k_conv3d_taps(ConvArgs a, int taps_per_gr
 
 // Forward / input gradient on a block tile (k_conv3d_blk): one CTA = 8 (x) x 16 (y) x ZT (z)
 // output voxels, i.e. ZT M-tiles of 128 rows (row r: x = x0 + (r & 7), y = y0 + (r >> 3)).  The
-// CTA loads its input block with a one-voxel halo (wrapped) into shared memory once, in three
-// copies shifted by dx = -1, 0, +1: copy s holds, for every 8-channel chunk, z and y of the
-// halo'd block, the 8 voxels x0 + s - 1 .. x0 + s + 6 as one 128-byte row (a core matrix of the
-// K-major layout: 8 rows of 16 bytes).  For a tap (dx, dy, dz) the A operand of an M-tile is copy
-// dx + 1 seen through a descriptor that starts dy + 1 rows and zt + dz + 1 planes in: the next y
-// is the next 128-byte row (stride between 8-row groups), the next channel chunk is one chunk
-// plane further (stride between K-adjacent core matrices).  Every core matrix stays 128-byte
-// aligned and no data moves per tap: thread 0 issues all 27 x CIN/16 MMAs of every M-tile back
-// to back into TMEM, with all 27 taps' weights resident, and one commit ends the CTA's work.
+// CTA loads its input block with a one-voxel halo (wrapped) into shared memory once: for every
+// 8-channel chunk, z and y of the halo'd block, a row of the 10 voxels x0 - 1 .. x0 + 8, 16 bytes
+// each.  Any 8 consecutive voxels of a row are a core matrix of the K-major layout (8 rows of 16
+// bytes; without swizzle a descriptor starts on any 16-byte boundary), so for a tap (dx, dy, dz) the
+// A operand of an M-tile is the block seen through a descriptor that starts dx + 1 voxels, dy + 1 rows
+// and zt + dz + 1 planes in: the next y is the next 160-byte row (stride between 8-row groups), the next
+// channel chunk is one chunk plane further (stride between K-adjacent core matrices).  No data moves
+// per tap: thread 0 issues all 27 x CIN/16 MMAs of every M-tile back to back into TMEM, with all 27
+// taps' weights resident, and one commit ends the CTA's work.  (Three copies of the block, one per dx, took
+// 166 of 207 KB at 48 -> 16 channels and left one CTA per SM: staging, MMAs and epilogue in sequence.)
 constexpr int kBlkX = 8, kBlkY = 16;
 constexpr int kBlkThreads = 256;   // 8 warps: staging in parallel, the epilogue's M-tiles split by warp quad
 
 template <int CIN, int COUT, int ZT>
-__host__ __device__ constexpr size_t blk_in_bytes() { return (size_t)3 * (CIN / 8) * (kBlkY + 2) * (ZT + 2) * 128; }
+__host__ __device__ constexpr size_t blk_in_bytes() { return (size_t)(CIN / 8) * (kBlkY + 2) * (ZT + 2) * (kBlkX + 2) * 16; }
 template <int CIN, int COUT, int ZT>
 __host__ __device__ constexpr size_t blk_smem_bytes() { return blk_in_bytes<CIN, COUT, ZT>() + (size_t)27 * COUT * CIN * 2; }
 
@@ -259,9 +260,9 @@ __global__ void __launch_bounds__(kBlkThreads) k_conv3d_blk(ConvArgs a)
     static_assert(CIN % 16 == 0 && COUT % 16 == 0 && ZT * COUT <= 256, "channel counts");
     constexpr int CH = CIN / 8;
     constexpr int BX = kBlkX + 2, BY = kBlkY + 2, BZ = ZT + 2;
-    constexpr uint32_t PLANE = BY * 128;             // one z plane of one chunk of one copy
-    constexpr uint32_t CHUNK = BZ * PLANE;           // one chunk of one copy (K-adjacent core matrices)
-    constexpr uint32_t COPY = CH * CHUNK;            // one shifted copy
+    constexpr uint32_t ROW = BX * 16;                // one row of the block (M-adjacent core matrices)
+    constexpr uint32_t PLANE = BY * ROW;             // one z plane of one chunk
+    constexpr uint32_t CHUNK = BZ * PLANE;           // one chunk (K-adjacent core matrices)
     constexpr uint32_t W_TAP = COUT * CIN * 2;       // bytes of one tap's weights
     constexpr uint32_t SBO_B = (CIN / 8) * 128;
     constexpr int NCOLS = ZT * COUT <= 32 ? 32 : (ZT * COUT <= 64 ? 64 : (ZT * COUT <= 128 ? 128 : 256));
@@ -287,8 +288,7 @@ __global__ void __launch_bounds__(kBlkThreads) k_conv3d_blk(ConvArgs a)
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         failed = 0;
     }
-    // halo'd input block: one global load per (voxel, chunk), chunks fastest (coalesced), stored
-    // into every shifted copy that contains the voxel (block x = bx is row position bx - s of copy s)
+    // halo'd input block: one global load per (voxel, chunk)
     // (batches of kBatch pieces per thread: all loads of a batch in flight before its stores)
     constexpr int kBatch = 8;
     constexpr int IN_TOT = BX * BY * BZ * CH, IN_IT = (IN_TOT + kBlkThreads - 1) / kBlkThreads;
@@ -308,12 +308,7 @@ __global__ void __launch_bounds__(kBlkThreads) k_conv3d_blk(ConvArgs a)
             const int idx = tid + (i0 + u) * kBlkThreads;
             if (i0 + u < IN_IT && idx < IN_TOT) {
                 const int bx = idx % BX, rest = idx / BX, c = rest % CH, row = rest / CH, by = row % BY, bz = row / BY;
-#pragma unroll
-                for (int sft = 0; sft < 3; ++sft) {
-                    const int xr = bx - sft;
-                    if (xr >= 0 && xr < kBlkX)
-                        *reinterpret_cast<uint4 *>(In + sft * COPY + c * CHUNK + bz * PLANE + by * 128 + xr * 16) = val[u];
-                }
+                *reinterpret_cast<uint4 *>(In + c * CHUNK + bz * PLANE + by * ROW + bx * 16) = val[u];
             }
         }
     }
@@ -350,13 +345,13 @@ __global__ void __launch_bounds__(kBlkThreads) k_conv3d_blk(ConvArgs a)
     if (tid == 0) {
         // every MMA's descriptors are the block's base descriptors plus a compile-time offset (in
         // 16-byte units of the start-address field; the block lies below 256 KB, so no carry)
-        const uint64_t da = smem_desc(smem_u32(In), CHUNK, 128), db = smem_desc(smem_u32(Wt), 128, SBO_B);
+        const uint64_t da = smem_desc(smem_u32(In), CHUNK, ROW), db = smem_desc(smem_u32(Wt), 128, SBO_B);
 #pragma unroll
         for (int zt = 0; zt < ZT; ++zt)
 #pragma unroll
             for (int tap = 0; tap < 27; ++tap) {
                 const int dz = tap / 9 - 1, dy = (tap / 3) % 3 - 1, dx = tap % 3 - 1;
-                const uint32_t ab = (uint32_t)(dx + 1) * COPY + (uint32_t)(zt + dz + 1) * PLANE + (uint32_t)(dy + 1) * 128;
+                const uint32_t ab = (uint32_t)(dx + 1) * 16 + (uint32_t)(zt + dz + 1) * PLANE + (uint32_t)(dy + 1) * ROW;
 #pragma unroll
                 for (int kk = 0; kk < CIN / 16; ++kk)
                     mma_bf16(tmem + zt * COUT, da + ((ab + kk * 2 * CHUNK) >> 4), db + ((tap * W_TAP + kk * 256) >> 4),
@@ -445,8 +440,10 @@ __global__ void __launch_bounds__(128) k_conv3d_wgrad_tc(WgradArgs a)
     constexpr int NCOLS = COUT <= 32 ? 32 : (COUT <= 64 ? 64 : 128);
     constexpr int KV = 128;                                // voxels per stage
     constexpr uint32_t A_BYTES = 128 * KV * 2, B_BYTES = COUT * KV * 2;
-    constexpr uint32_t SBO = (KV / 8) * 128;
-    constexpr uint32_t IDESC = idesc_bf16(128, COUT);
+    // operands with channels contiguous, as they lie in memory: 8 voxels x 8 channels per core matrix, the
+    // channel chunks of 8 voxels side by side, then the next 8 voxels
+    constexpr uint32_t A_KB = 128 / 8 * 128, B_KB = COUT / 8 * 128;   // bytes per 8 voxels
+    constexpr uint32_t IDESC = idesc_bf16(128, COUT, true);
     extern __shared__ __align__(1024) unsigned char smem[];
     unsigned char *Abuf = smem;
     unsigned char *Bbuf = smem + 2 * A_BYTES;
@@ -472,6 +469,45 @@ __global__ void __launch_bounds__(128) k_conv3d_wgrad_tc(WgradArgs a)
     const uint32_t tmem = tmem_slot;
     const int chunk0 = blockIdx.y * a.chunks_per_cta;
     const int nchunks = min(a.chunks_per_cta, nvox / KV - chunk0);
+    // Pipeline: a stage's operands are loaded into registers right after the previous stage's MMAs are issued
+    // and stored once their buffer is free.  Which voxel feeds (tap, row) is tabulated one stage ahead, one voxel per
+    // thread, so a stage costs one coordinate division per thread instead of one per 16-byte piece.
+    // Pieces are mapped by piece_rc: 8 lanes fill one core matrix, a warp reads 64 contiguous bytes of each of 8 voxels.
+    constexpr int CHI = CIN / 8, A_IT = TPG * CHI, CHO = COUT / 8, B_IT = CHO;   // pieces per thread (KV = threads)
+    static_assert(KV == 128, "one voxel of the table per thread");
+    __shared__ int nbt[2][TPG][KV];   // source voxel of each tap of the group
+    auto table = [&](int s) {
+        const int v = (chunk0 + s) * KV + tid;
+        const int r = v / nx, i = v - r * nx, k = r / ny, j = r - k * ny;
+#pragma unroll
+        for (int tl = 0; tl < TPG; ++tl) {
+            const int tap = min(tap0 + tl, 26);
+            const int dz = tap / 9 - 1, dy = (tap / 3) % 3 - 1, dx = tap % 3 - 1;
+            nbt[s & 1][tl][tid] = wrapi(i + dx, nx) + nx * (wrapi(j + dy, ny) + ny * wrapi(k + dz, nz));
+        }
+    };
+    uint4 av[A_IT], bv[B_IT];
+    auto load = [&](int s) {
+#pragma unroll
+        for (int u = 0; u < A_IT; ++u) {
+            const int tl = u / CHI;
+            int kv, c;
+            piece_rc<CHI>(tid + (u - tl * CHI) * 128, kv, c);
+            if (tl < ntap)
+                av[u] = *reinterpret_cast<const uint4 *>(a.x + (size_t)nbt[s & 1][tl][kv] * a.xcs + a.xc0 + c * 8);
+        }
+#pragma unroll
+        for (int u = 0; u < B_IT; ++u) {
+            int kv, c;
+            piece_rc<CHO>(tid + u * 128, kv, c);
+            bv[u] = *reinterpret_cast<const uint4 *>(a.dy + (size_t)((chunk0 + s) * KV + kv) * a.dcs + a.dc0 + c * 8);
+        }
+    };
+    if (nchunks > 0) {
+        table(0);
+        __syncthreads();
+        load(0);
+    }
     int issued = 0;
     for (int s = 0; s < nchunks; ++s) {
         const int buf = s & 1;
@@ -482,71 +518,27 @@ __global__ void __launch_bounds__(128) k_conv3d_wgrad_tc(WgradArgs a)
         }
         unsigned char *A = Abuf + buf * A_BYTES;
         unsigned char *B = Bbuf + buf * B_BYTES;
-        const int vbase = (chunk0 + s) * KV;
         // A rows r = tl * CIN + ci (tap tl of the group, input channel ci), K = voxel kv
-        for (int idx = tid; idx < 128 * (KV / 8); idx += 128) {   // zero unused rows first
-            int r = idx / (KV / 8), kc = idx % (KV / 8);
-            if (r >= ntap * CIN) *reinterpret_cast<uint4 *>(A + (r >> 3) * SBO + kc * 128 + (r & 7) * 16) = make_uint4(0, 0, 0, 0);
+        if (ntap * CIN < 128 && s < 2)   // unused rows: zero, once per buffer
+            for (int idx = tid; idx < KV * 16; idx += 128) {
+                const int kv = idx & 127, m = idx >> 7;
+                if (m * 8 >= ntap * CIN)
+                    *reinterpret_cast<uint4 *>(A + (kv >> 3) * A_KB + m * 128 + (kv & 7) * 16) = make_uint4(0, 0, 0, 0);
+            }
+#pragma unroll
+        for (int u = 0; u < A_IT; ++u) {
+            const int tl = u / CHI;
+            int kv, c;
+            piece_rc<CHI>(tid + (u - tl * CHI) * 128, kv, c);
+            if (tl < ntap) *reinterpret_cast<uint4 *>(A + (kv >> 3) * A_KB + (tl * CHI + c) * 128 + (kv & 7) * 16) = av[u];
         }
-        // (batches of 8 pieces per thread: all loads of a batch in flight before its stores)
-        constexpr int A_IT = TPG * KV * (CIN / 8) / 128;
-        const int a_tot = ntap * KV * (CIN / 8);
-        for (int i0 = 0; i0 < A_IT; i0 += 8) {
-            uint4 val[8];
 #pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                const int idx = tid + (i0 + u) * 128;
-                if (i0 + u < A_IT && idx < a_tot) {
-                    const int c = idx % (CIN / 8), kv = (idx / (CIN / 8)) % KV, tl = idx / ((CIN / 8) * KV);
-                    const int tap = tap0 + tl;
-                    const int dz = tap / 9 - 1, dy = (tap / 3) % 3 - 1, dx = tap % 3 - 1;
-                    const int v = vbase + kv;
-                    const int i = v % nx, j = (v / nx) % ny, k = v / (nx * ny);
-                    const int nb = wrapi(i + dx, nx) + nx * (wrapi(j + dy, ny) + ny * wrapi(k + dz, nz));
-                    val[u] = *reinterpret_cast<const uint4 *>(a.x + (size_t)nb * a.xcs + a.xc0 + c * 8);
-                }
-            }
-#pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                const int idx = tid + (i0 + u) * 128;
-                if (i0 + u < A_IT && idx < a_tot) {
-                    const int c = idx % (CIN / 8), kv = (idx / (CIN / 8)) % KV, tl = idx / ((CIN / 8) * KV);
-                    const __nv_bfloat16 *e = reinterpret_cast<const __nv_bfloat16 *>(&val[u]);
-#pragma unroll
-                    for (int q = 0; q < 8; ++q) {
-                        const int r = tl * CIN + c * 8 + q;
-                        *reinterpret_cast<__nv_bfloat16 *>(A + (r >> 3) * SBO + (kv >> 3) * 128 + (r & 7) * 16 +
-                                                           (kv & 7) * 2) = e[q];
-                    }
-                }
-            }
+        for (int u = 0; u < B_IT; ++u) {
+            int kv, c;
+            piece_rc<CHO>(tid + u * 128, kv, c);
+            *reinterpret_cast<uint4 *>(B + (kv >> 3) * B_KB + c * 128 + (kv & 7) * 16) = bv[u];
         }
-        constexpr int B_IT = (KV * (COUT / 8) + 127) / 128;
-        for (int i0 = 0; i0 < B_IT; i0 += 8) {
-            uint4 val[8];
-#pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                const int idx = tid + (i0 + u) * 128;
-                if (i0 + u < B_IT && idx < KV * (COUT / 8)) {
-                    const int c = idx % (COUT / 8), kv = idx / (COUT / 8);
-                    val[u] = *reinterpret_cast<const uint4 *>(a.dy + (size_t)(vbase + kv) * a.dcs + a.dc0 + c * 8);
-                }
-            }
-#pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                const int idx = tid + (i0 + u) * 128;
-                if (i0 + u < B_IT && idx < KV * (COUT / 8)) {
-                    const int c = idx % (COUT / 8), kv = idx / (COUT / 8);
-                    const __nv_bfloat16 *e = reinterpret_cast<const __nv_bfloat16 *>(&val[u]);
-#pragma unroll
-                    for (int q = 0; q < 8; ++q) {
-                        const int r = c * 8 + q;
-                        *reinterpret_cast<__nv_bfloat16 *>(B + (r >> 3) * SBO + (kv >> 3) * 128 + (r & 7) * 16 +
-                                                           (kv & 7) * 2) = e[q];
-                    }
-                }
-            }
-        }
+        if (s + 1 < nchunks) table(s + 1);
         fence_proxy_async();
         fence_before_sync();
         __syncthreads();
@@ -555,11 +547,12 @@ __global__ void __launch_bounds__(128) k_conv3d_wgrad_tc(WgradArgs a)
             const uint32_t a0 = smem_u32(A), b0 = smem_u32(B);
 #pragma unroll
             for (int kk = 0; kk < KV / 16; ++kk)
-                mma_bf16(tmem, smem_desc(a0 + kk * 256, 128, SBO), smem_desc(b0 + kk * 256, 128, SBO), IDESC,
+                mma_bf16(tmem, smem_desc(a0 + kk * 2 * A_KB, A_KB, 128), smem_desc(b0 + kk * 2 * B_KB, B_KB, 128), IDESC,
                          (s > 0 || kk > 0) ? 1u : 0u);
             mma_commit(&mbar[buf]);
         }
         ++issued;
+        if (s + 1 < nchunks) load(s + 1);   // in flight during the next buffer wait
     }
     if (tid == 0 && issued > 0) {
         const int last = issued - 1;
@@ -626,7 +619,11 @@ int launch_fwd(const ConvArgs &a, int nvox, float *ws, cudaStream_t st)
     constexpr int ZT = 2;
     constexpr size_t bsm = blk_smem_bytes<CIN, COUT, ZT>();
     if constexpr (bsm <= 220 * 1024) {
-        if (a.n0 % kBlkX == 0 && a.n1 % kBlkY == 0 && a.n2 % ZT == 0) {
+        // the largest layers (64 -> 32, 32 -> 96: block and weights near the limit) only on grids of at
+        // least 96 blocks: below, the split taps spread the work over more SMs
+        constexpr bool large = (CIN == 64 && COUT == 32) || (CIN == 32 && COUT == 96);
+        const long long tiles = (long long)(a.n0 / kBlkX) * (a.n1 / kBlkY) * (a.n2 / ZT);
+        if (a.n0 % kBlkX == 0 && a.n1 % kBlkY == 0 && a.n2 % ZT == 0 && (!large || tiles >= 96)) {
             static bool attr_blk = false;
             if (!attr_blk) {
                 if (cudaFuncSetAttribute(k_conv3d_blk<CIN, COUT, ZT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -674,7 +671,9 @@ int launch_wgrad(const WgradArgs &a0, int nvox, cudaStream_t st)
     WgradArgs a = a0;
     const int chunks = nvox / 128;
     const int groups = (27 + TPG - 1) / TPG;
-    // enough CTAs to fill the GPU a few times over: split the voxel chunks
+    // four CTAs per SM in all (two resident): the voxel chunks are split.  Fewer, longer reductions would save
+    // atomics, but the FP32 error of a partial grows with its length (32^3, 96 -> 32: 5.6e-7 with 12 chunks
+    // of 128 voxels per CTA, above 1e-6 with 24)
     int splits = std::max(1, std::min(chunks, (152 * 4 + groups - 1) / groups));
     a.chunks_per_cta = (chunks + splits - 1) / splits;
     splits = (chunks + a.chunks_per_cta - 1) / a.chunks_per_cta;

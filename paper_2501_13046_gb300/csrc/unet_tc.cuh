@@ -23,12 +23,16 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo, uint3
     return d;                 // base offset 0, no swizzle
 }
 
-// Instruction descriptor of kind::f16: D = F32, A = B = BF16, both K-major, shape M x N.
-__host__ __device__ constexpr uint32_t idesc_bf16(int M, int N)
+// Instruction descriptor of kind::f16: D = F32, A = B = BF16, shape M x N; both operands K-major, or
+// (mn_major) both with M / N contiguous: an 8 x 8 core matrix is then 8 rows of K, 16 bytes of 8
+// consecutive M (N) values each, and the shared-memory descriptor's lbo is the distance between core matrices
+// adjacent in K, sbo between those adjacent in M (N).
+__host__ __device__ constexpr uint32_t idesc_bf16(int M, int N, bool mn_major = false)
 {
     return (1u << 4)                       // D format F32
            | (1u << 7)                     // A format BF16
            | (1u << 10)                    // B format BF16
+           | (mn_major ? 3u << 15 : 0u)    // A, B transposed
            | ((uint32_t)(N >> 3) << 17)    // N / 8
            | ((uint32_t)(M >> 4) << 24);   // M / 16
 }
