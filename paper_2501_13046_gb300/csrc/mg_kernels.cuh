@@ -948,12 +948,6 @@ __global__ void __launch_bounds__(256) k_prolong_add(Geo g, Geo gc, const T *__r
     }
 }
 
-template <typename T>
-__device__ __noinline__ T robin_ratio_call(const Geo &g, int bi, int bj, int bk, int gi, int gj, int gk)
-{
-    return robin_ratio<T>(g, bi, bj, bk, gi, gj, gk);
-}
-
 // k_prolong_add for periodic and Robin boxes, one thread per coarse cell and field: its 2 x 2 x 2 fine cells share the
 // 27 coarse values around it (3.4 reads per fine cell and field instead of 8), combined axis by axis.  A thread's
 // x pairs are one cell of each colour at the same storage place, so fine accesses are contiguous over a
@@ -980,6 +974,21 @@ __global__ void __launch_bounds__(128) k_prolong_blocks(Geo g, Geo gc, const T *
                 else q = min(max(q, 0), n - 1);
                 p[a][d] = q;
             }
+        // squared coordinates of those places and of the cells themselves (the Robin ratio is |x_b| / |x_g|)
+        T sb[3][3], sg[3][3];
+        if constexpr (BC != BC_PERIODIC)
+#pragma unroll
+            for (int a = 0; a < 3; ++a)
+#pragma unroll
+                for (int d = 0; d < 3; ++d) {
+                    auto centre = [&](int i) {
+                        if constexpr (std::is_same<T, float>::value) return gc.lof[a] + ((float)i + 0.5f) * gc.hf[a];
+                        else return gc.lo[a] + (i + 0.5) * gc.h[a];
+                    };
+                    const T xb = centre(p[a][d]), xg = centre(at[a] + d - 1);
+                    sb[a][d] = xb * xb;
+                    sg[a][d] = xg * xg;
+                }
         const bool edge = BC != BC_PERIODIC && (I == 0 || J == 0 || K == 0 || I == gc.n[0] - 1 || J == gc.n[1] - 1 || K == gc.n[2] - 1);
         auto place = [&](int x, int y, int z) -> unsigned {   // (31-bit cell counts)
             const unsigned lin = (unsigned)x + ncx * ((unsigned)y + ncy * (unsigned)z);
@@ -1009,8 +1018,16 @@ __global__ void __launch_bounds__(128) k_prolong_blocks(Geo g, Geo gc, const T *
 #pragma unroll
                     for (int x = 0; x < 3; ++x) {
                         v[x] = e[place(p[0][x], p[1][y], p[2][z])];
-                        if (edge && (I + x - 1 != p[0][x] || J + y - 1 != p[1][y] || K + z - 1 != p[2][z]))
-                            v[x] *= robin_ratio_call<T>(gc, p[0][x], p[1][y], p[2][z], I + x - 1, J + y - 1, K + z - 1);
+                        if constexpr (BC != BC_PERIODIC) {
+                            if (edge) {   // (as robin_ratio; 1 where nothing was clamped)
+                                const T A = sb[0][x] + sb[1][y] + sb[2][z], B = sg[0][x] + sg[1][y] + sg[2][z];
+                                T ratio;
+                                if constexpr (std::is_same<T, float>::value) ratio = A * rsqrtf(A * B);
+                                else ratio = sqrt(A / B);
+                                const bool ghost = I + x - 1 != p[0][x] || J + y - 1 != p[1][y] || K + z - 1 != p[2][z];
+                                v[x] *= ghost ? ratio : (T)1;
+                            }
+                        }
                     }
                     const T x0 = (T)0.75 * v[1] + (T)0.25 * v[0], x1 = (T)0.75 * v[1] + (T)0.25 * v[2];
                     if (y == 0) {
