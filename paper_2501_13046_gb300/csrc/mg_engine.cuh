@@ -61,6 +61,16 @@ mg_status launch_tile(mg_ctx *x, const LevelBufs &L, const TileCoef<T> &tc, cons
     return MG_OK;
 }
 
+// Before the first work of an iteration on a level below the finest: its coefficients come from the side branch.
+inline mg_status wait_coefficients(mg_ctx *x)
+{
+    if (x->coef_pending) {
+        CK(cudaStreamWaitEvent(x->stream, x->ev_coef, 0));
+        x->coef_pending = false;
+    }
+    return MG_OK;
+}
+
 // Residual of level l's current correction, restricted to the right-hand side of level l + 1.
 template <typename T, int ORDER, int BC>
 mg_status enqueue_restrict(mg_ctx *x, int l)
@@ -219,6 +229,7 @@ mg_status enqueue_cycle(mg_ctx *x, int l, bool zero)
 {
     const int Lc = x->nlev - 1;
     LevelBufs &L = x->lev[l];
+    if (l > 0 || l == x->cluster || (x->fused && l == Lc - 1)) CKS(wait_coefficients(x));
     if (l == Lc) {   // the coarse solve writes the whole correction
         L.curB = 0;
         return enqueue_coarse<T, ORDER, BC>(x, Lc);
@@ -325,17 +336,26 @@ inline size_t gj_smem(int m)
     return b <= kMaxCoarseSmem ? b : 0;
 }
 
-// Inverse of the coarsest psi row for this outer iteration (its coefficients were just restricted),
-// on a parallel branch: the one-CTA inversion overlaps the first cycle's descent, and the first
-// coarse solve of the iteration waits for it (enqueue_coarse).
+// The coarser levels' psi-row coefficients and the inverse of the coarsest psi row for this outer iteration, on a
+// parallel branch: the finest level's first sweeps need neither.  The first work on a coarser level waits for
+// the coefficients (wait_coefficients), the first coarse solve for the inverse (join_pending).
 template <typename T, int ORDER, int BC>
-mg_status enqueue_dense_psi_inverse(mg_ctx *x)
+mg_status enqueue_coefficients(mg_ctx *x)
 {
+    CK(cudaEventRecord(x->ev_fork, x->stream));
+    CK(cudaStreamWaitEvent(x->side, x->ev_fork, 0));
+    for (int l = 1; l < x->nlev; ++l) {
+        LevelBufs &C = x->lev[l];
+        k_restrict_mean<T><<<grid_for(C.N), kThreads, 0, x->side>>>(x->lev[l - 1].geo, C.geo, (const T *)x->lev[l - 1].c,
+                                                                   (T *)C.c, 2, C.split);
+    }
+    CK(cudaGetLastError());
+    CK(cudaEventRecord(x->ev_coef, x->side));
+    x->coef_pending = true;
+    if (!x->dense) return MG_OK;
     LevelBufs &C = x->lev[x->nlev - 1];
     const int periodic = x->cfg.bc == MG_BC_PERIODIC;
     Coef<T> cf = make_coef<T>(C.geo, x->cfg.order);
-    CK(cudaEventRecord(x->ev_fork, x->stream));
-    CK(cudaStreamWaitEvent(x->side, x->ev_fork, 0));
     with_bc<BC>([&](auto B) {
         k_dense_psi_assemble<T, T, ORDER, decltype(B)::value><<<1, 512, 0, x->side>>>(C.geo, cf, (const T *)C.c,
                                                                                     (T *)x->gj, periodic);
@@ -377,13 +397,7 @@ mg_status engine_dense_setup(mg_ctx *x)
 template <typename T, int ORDER, int BC>
 mg_status enqueue_iteration(mg_ctx *x)
 {
-    for (int l = 1; l < x->nlev; ++l) {
-        LevelBufs &C = x->lev[l];
-        k_restrict_mean<T><<<grid_for(C.N), kThreads, 0, x->stream>>>(x->lev[l - 1].geo, C.geo,
-                                                                       (const T *)x->lev[l - 1].c, (T *)C.c, 2, C.split);
-    }
-    CK(cudaGetLastError());
-    if (x->dense) CKS(enqueue_dense_psi_inverse<T, ORDER, BC>(x));
+    if (x->nlev > 1) CKS(enqueue_coefficients<T, ORDER, BC>(x));
     LevelBufs &L0 = x->lev[0];
     if (x->zsolve) {   // z = L^-1 (dF/dK^2) in the inner form: the cycles on zrhs, its means
         void *f = L0.f;

@@ -1269,22 +1269,6 @@ static __global__ void __launch_bounds__(256) k_flag_nonfinite(const double *__r
     if (__syncthreads_or(bad) && threadIdx.x == 0) atomicOr(flag, 1u);
 }
 
-// Final single-block reduction of per-block partial maxima: partial[b * NV + a].
-template <int NV>
-__global__ void k_finalize_max(const double *__restrict__ partial, int nblocks, double *__restrict__ out)
-{
-    double v[NV];
-#pragma unroll
-    for (int a = 0; a < NV; ++a) v[a] = 0.0;
-    for (int b = threadIdx.x; b < nblocks; b += blockDim.x)
-#pragma unroll
-        for (int a = 0; a < NV; ++a) v[a] = fmax(v[a], partial[b * NV + a]);
-    double r[NV];
-    block_max<NV>(v, r);
-    if (threadIdx.x == 0)
-        for (int a = 0; a < NV; ++a) out[a] = r[a];
-}
-
 // Sums of 4 contiguous fields (block partials); with means != nullptr the last block also forms
 // means[a] = sum_a / N (ticket: its finalize_last counter).  Fields of a multiple of 4 cells (every
 // grid with more than one level) are read 16 bytes at a time.  128^3 FP32: 35 -> 9 us.

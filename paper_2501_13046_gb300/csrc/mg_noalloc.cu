@@ -44,9 +44,9 @@ mg_status scratch_address(double **out)
     return MG_OK;
 }
 
-// Block partial maxima of |H| and |M_i| (nothing else is written).
+// Maxima of |H| and |M_i|, finished in the last block.
 __global__ void __launch_bounds__(256) k_noalloc_norms(Geo g, const double *__restrict__ u,
-                                                       const double *__restrict__ R, const Scalars *__restrict__ s,
+                                                       const double *__restrict__ R, Scalars *s,
                                                        double *__restrict__ partial)
 {
     const size_t N = (size_t)g.n[0] * g.n[1] * g.n[2];
@@ -70,6 +70,7 @@ __global__ void __launch_bounds__(256) k_noalloc_norms(Geo g, const double *__re
     block_max<4>(mx, r);
     if (threadIdx.x == 0)
         for (int a = 0; a < 4; ++a) partial[blockIdx.x * 4 + a] = r[a];
+    finalize_last<4, true>(partial, gridDim.x, s->norms, &s->ticket[1]);
 }
 
 mg_status check_config(const mg_config *c)
@@ -160,7 +161,6 @@ extern "C" mg_status mg_residual_norms_noalloc(const mg_config *cfg, const doubl
     }
     CK(attr);
     k_noalloc_norms<<<g1, kThreads, 0, st>>>(g, u, R, sc, partial);
-    k_finalize_max<4><<<1, 256, 0, st>>>(partial, g1, sc->norms);
     CK(cudaGetLastError());
     Scalars h;
     CK(cudaMemcpyAsync(&h, sc, sizeof(Scalars), cudaMemcpyDeviceToHost, st));
