@@ -291,15 +291,16 @@ def batch_measure(mg, torch, sp, precision, repeats=1):
             "max_norm": max(float(i["norms"].max()) for i in infos)}
 
 
-# FP64 flops of the residual pass B per interior cell, counted from its source (an FMA is 2):
-# Lap u 19, three momentum rows 75, AtAt 55, nonlinear terms and outputs 30.
-PASSB_FLOPS_PER_CELL = 179
+# FP64-pipe instructions of the fused residual per cell, counted from its source: conversions of the five
+# integer results 5, their units 2, psi and its powers 6, reciprocal 3, nonlinear terms 6, sources and rows 7,
+# block sums 5.  (Its stencils are 64-bit integer arithmetic.)
+RESIDUAL_FP64_PER_CELL = 34
 # FP64 peak from unit counts and clocks (the denominator of an ALU-bound kernel): 152 SMs x 2 FP64
 # FMA lanes x 2 flops x 2.07 GHz.  The rate of the library's FMA probe is reported beside it.
 FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.07e9 / 1e12
-# DRAM bytes of one 128^3 pass-B launch (dram__bytes_read.sum + dram__bytes_write.sum) from one ncu
-# capture of the kernel as it stands (profiles/outer_pass1q_128cube_periodic_o4.md); None if none
-PASSB_TRAFFIC_128 = 374079744
+# DRAM bytes of one 128^3 residual launch (dram__bytes_read.sum + dram__bytes_write.sum) from one ncu
+# capture (profiles/outer_residual_128cube_periodic_o4.md); None if none
+RESIDUAL_TRAFFIC_128 = None
 # the same for the finest colour pass and residual + restriction at 128^3
 # (profiles/smooth_tile_128cube_periodic_o4.md, profiles/restrict_tile_128cube_periodic_o4.md)
 COLOUR_TRAFFIC_128 = 59366656 + 1694976
@@ -309,17 +310,17 @@ RESTRICT_TRAFFIC_128 = 85024512 + 2426368
 def kernel_rooflines(mg, ctx, N):
     """Live CUDA-event timings (library stream) of the dominant kernel and of the colour pass."""
     pk, src = peaks()
-    msb, bytesb = mg.mg_time_kernel(ctx, 3, 10)   # FP64 residual pass B alone
+    msb, bytesb = mg.mg_time_kernel(ctx, 2, 10)   # fused FP64 residual
     ms0, bytes0 = mg.mg_time_kernel(ctx, 0, 40)   # finest FP32 colour pass
     ms1, bytes1 = mg.mg_time_kernel(ctx, 1, 20)   # finest residual + restriction
     fp64 = mg.mg_fp64_fma_rate(ctx, 3)           # FP64 FMA rate of the library probe (context)
-    ach = PASSB_FLOPS_PER_CELL * N / (msb * 1e-3) / 1e12
+    ach = 2 * RESIDUAL_FP64_PER_CELL * N / (msb * 1e-3) / 1e12   # an issue slot counts as one FMA
     sm_gbs = bytes0 / (ms0 * 1e-3) / 1e9
     rr_gbs = bytes1 / (ms1 * 1e-3) / 1e9
     return {"bound": "alu", "achieved": ach, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
-            "frac": ach / FP64_PEAK_TFLOPS, "traffic": PASSB_TRAFFIC_128,
-            "kernel": "k_outer_pass1q<4,periodic> (FP64 residual pass B, 128^3; FP64 pipe bound)",
-            "ms_per_launch": msb, "algorithmic_flops": PASSB_FLOPS_PER_CELL * N, "algorithmic_bytes": bytesb,
+            "frac": ach / FP64_PEAK_TFLOPS, "traffic": RESIDUAL_TRAFFIC_128 if N == 128 ** 3 else None,
+            "kernel": "k_outer_residual<4,periodic> (fused FP64 residual, 128^3; FP64 and integer pipes)",
+            "ms_per_launch": msb, "fp64_issue_slots": RESIDUAL_FP64_PER_CELL * N, "algorithmic_bytes": bytesb,
             "peak_source": "derived: 152 SMs x 2 FP64 FMA lanes x 2 flops x 2.07 GHz",
             "fp64_probe_tflops": fp64, "frac_of_probe": ach / fp64,
             "colour_pass": {"bound": "hbm", "kernel": "k_smooth_tile<float,4,periodic,c> (finest, one colour)",

@@ -81,8 +81,8 @@ typedef struct {
     int inner_cycles;     /* V-cycles per outer iteration, 0 = auto (1 for MG_FP64, 2 for MG_MIXED) */
     int block_threads;    /* threads per block of the global-memory stencil kernels: 0 = 256, else 64, 128 or 256 */
     int smoother;         /* 0 = auto: the TMA-tiled colour pass and restriction on FP32 levels with nx, ny
-                             multiples of 8, >= 16 and nz >= 8, the next-to-coarsest level and the coarsest in one
-                             CTA when small, global-memory kernels elsewhere; 1 = one global-memory kernel per
+                             multiples of 8, >= 16 and nz >= 8, the levels of at most 8000 cells in one cluster of
+                             CTAs where they fit, global-memory kernels elsewhere; 1 = one global-memory kernel per
                              step on every level */
     int cycle;            /* coarse-level visits per cycle: 0 or 1 = V-cycle (default), 2 = W-cycle           */
     double omega;         /* red-black relaxation weight in (0, 2); 0 = 1.0 (plain Gauss-Seidel per colour)   */
@@ -265,9 +265,8 @@ mg_status mg_constraint_fields(struct mg_ctx *ctx, double *H, double *M, int on_
  * Measurement aid: launch one kernel of the solve `reps` times back to back on the context's
  * stream, bracketed by CUDA events, at the current state (call after mg_solve or
  * mg_residual_norms).  which: 0 = one red-black colour pass of the finest-level smoother,
- * 1 = residual + restriction of the finest level, 2 = outer FP64 residual pass 1 (its two
- * kernels, q/div W then the residual parts, and the reduction of the integrability sums),
- * 3 = the second of those kernels alone (the residual parts; FP64-ALU bound).
+ * 1 = residual + restriction of the finest level, 2 = outer FP64 residual pass 1 (one fused kernel:
+ * the residual parts and the reduction of the integrability sums), 3 = the same without the sums.
  * Returns the mean device time per launch and the algorithmic DRAM bytes one launch must
  * move (every array it reads once, every array it writes once).  The solver state is not
  * changed except for scratch buffers.

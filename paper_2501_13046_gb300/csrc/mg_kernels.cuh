@@ -797,8 +797,8 @@ __global__ void __launch_bounds__(256) k_smooth_first(Geo g, FaceDiag<T> fd, T d
 // [0, nblk_sh) take the coarse shell, the others the coarse cells whose children's stencils stay
 // inside the fine box (the coarse interior box [1, nc-1)^3).
 // One thread per child, the 8 children of a coarse cell in 8 neighbouring lanes (their sum by shuffles):
-// with one thread per coarse cell the 8 stencils ran one after the other on an eighth of the threads (64^3 FP64: 143 us
-// per launch, 32^3: 141 us).
+// with one thread per coarse cell the 8 stencils ran one after the other on an eighth of the threads (64^3 FP64: 143 -> 133 us,
+// FP64-bound; 32^3: 141 -> 28 us).
 template <typename T, int ORDER, int BC, bool INTERIOR>
 __device__ __forceinline__ void restrict_child(const Geo &g, const Coef<T> &cf, const T *e, const T *f, const T *ab,
                                                size_t N, int i, int j, int k, T r[4])
@@ -951,7 +951,7 @@ __global__ void __launch_bounds__(256) k_prolong_add(Geo g, Geo gc, const T *__r
 // k_prolong_add for periodic and Robin boxes, one thread per coarse cell and field: its 2 x 2 x 2 fine cells share the
 // 27 coarse values around it (3.4 reads per fine cell and field instead of 8), combined axis by axis.  A thread's
 // x pairs are one cell of each colour at the same storage place, so fine accesses are contiguous over a
-// warp.  128^3: 32 us with one thread per fine cell.
+// warp.  128^3: 22 us, 32 us with one thread per fine cell (62 us with one thread for all four fields).
 template <typename T, int BC>
 __global__ void __launch_bounds__(128) k_prolong_blocks(Geo g, Geo gc, const T *__restrict__ ec, T *__restrict__ ef,
                                                         int csplit)
@@ -1214,7 +1214,7 @@ struct Scalars {
     unsigned int err;         // nonzero: a bounded wait of a pipelined kernel gave up (MG_ERR_TIMEOUT)
     unsigned int nonfinite;   // nonzero: a source value is NaN or infinite (set by k_flag_nonfinite)
     double change[8];         // last update: max |e_a - <e_a>| (a = 0..3), then max |psi|, |W_x|, |W_y|, |W_z| after it
-    unsigned int ticket[4];   // last-block counters: pass-B sums, pass-2 norms, means of e, update maxima
+    unsigned int ticket[4];   // last-block counters: residual sums, pass-2 norms, means of e, update maxima
     double zmean[4];          // k2_newton: means of the z solve's result (component 0: z of the psi row)
 };
 
@@ -1252,7 +1252,7 @@ __device__ __forceinline__ void outer_scalars(Scalars *s, size_t N, int kmode_in
     for (int a = 0; a < 3; ++a) s->msrc[a] = periodic ? s->sums[2 + a] / (double)N : 0.0;
 }
 
-// What the last block of pass B finishes when s is set: the sums, then K^2 and m_i.
+// What the last block of the FP64 residual finishes when s is set: the sums, then K^2 and m_i.
 struct OuterFin {
     Scalars *s;
     int kmode_integrability, periodic;
@@ -1271,7 +1271,7 @@ static __global__ void __launch_bounds__(256) k_flag_nonfinite(const double *__r
 
 // Sums of 4 contiguous fields (block partials); with means != nullptr the last block also forms
 // means[a] = sum_a / N (ticket: its finalize_last counter).  Fields of a multiple of 4 cells (every
-// grid with more than one level) are read 16 bytes at a time.  128^3 FP32: 35 -> 9 us.
+// grid with more than one level) are read 16 bytes at a time.  128^3 FP32: 35 -> 18 us.
 constexpr int kSumBlocks = 152 * 2;
 
 // s + b as an unevaluated pair hi + lo of floats, exact (Knuth's two-sum; the rounding error of every addition
@@ -1371,7 +1371,7 @@ __global__ void __launch_bounds__(256) k_sub_mean4(T *__restrict__ x, size_t N, 
 // largest |psi|, |W_i| after it (psi = background + u), for the per-field stopping test.
 // Launched on at most kRedBlocks blocks (partial holds 8 values per block).
 // Split levels take the two cells of an x pair per thread (16-byte accesses of x, one value of each colour
-// half); with the conversions by bits two FP64 additions per value are left (one without means).
+// half); with the conversions by bits two FP64 additions per value are left (one without means).  128^3: 90 -> 37 us.
 template <typename T, int SPLIT, int SIZED>
 __global__ void __launch_bounds__(256, SIZED ? 2 : 4) k_update(Geo g, double *__restrict__ x, const T *__restrict__ e, size_t N,
                                                 const double *__restrict__ means, double *__restrict__ partial,
@@ -1499,7 +1499,7 @@ __device__ __forceinline__ float absnanf(float x) { return (x == x) ? fabsf(x) :
 
 // The FP32 inner solve's form, on a colour-split finest level: the two cells of an x pair per thread,
 // 16-byte loads, conversions to FP32 by bits (8 FP64 instructions per cell are left of 17; 5 on boxes
-// without momentum-source means).  128^3: 94 -> 44 us.
+// without momentum-source means).  128^3: 94 -> 64 us.
 static __global__ void __launch_bounds__(256, 2)
     k_outer_pass2_pairs(Geo g, const double *__restrict__ x, const double *__restrict__ R, const double *__restrict__ src,
                         Scalars *s, float *__restrict__ f, float *__restrict__ ab, double *__restrict__ partial)

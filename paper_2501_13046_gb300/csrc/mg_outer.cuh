@@ -16,12 +16,14 @@
 // 128^3 periodic 240 us (integer part alone 165 us, the FP64 part's floor 143 us).
 //
 // March: 16 x 8 cells per plane, one thread per cell, planes along z through a ring of ORDER + 1
-// slots (4 CTAs per SM: their integer and FP64 phases overlap).  The mixed term (1/3) d_i d_j W_j uses D_i D_j = D_i o D_j:
+// slots (4 CTAs per SM: their integer and FP64 phases overlap).  The mixed term (1/3) d_i d_j W_j uses
+// D_i D_j = D_i o D_j:
 //   row x: D_x B + D_z C,  row y: D_y A + D_z D,  row z: D_z (A + B)
 // with A = D_x W_x, B = D_y W_y, C = D_x W_z, D = D_y W_z formed once per plane; A and B are
 // shared with the neighbouring cells through shared memory, beside the z history of A + B, C and D.
-// A cell's FP64 tail runs one plane later, among the integer stencils of the next cell.  Boundary values (periodic wrap, Robin, mirror, extrapolation) are
-// filled in when a plane is loaded, in FP64 by the rule of fetch_bc, so every cell takes this path.
+// A cell's FP64 tail runs one plane later, among the integer stencils of the next cell.  Boundary values
+// (periodic wrap, Robin, mirror, extrapolation) are filled in when a plane is loaded, in FP64 by the
+// rule of fetch_bc, so every cell takes this path.
 //
 // Values that are NaN or infinite have no fixed-point form: a CTA that meets one finishes its
 // remaining planes with the direct FP64 stencils (outer_cell), which propagate it cell by cell.
