@@ -291,16 +291,15 @@ def batch_measure(mg, torch, sp, precision, repeats=1):
             "max_norm": max(float(i["norms"].max()) for i in infos)}
 
 
-# FP64-pipe instructions of the fused residual per cell, counted from its source: conversions of the five
-# integer results 5, their units 2, psi and its powers 6, reciprocal 3, nonlinear terms 6, sources and rows 7,
-# block sums 5.  (Its stencils are 64-bit integer arithmetic.)
-RESIDUAL_FP64_PER_CELL = 34
+# FP64-pipe instructions of the fused residual per cell, from one ncu capture at 128^3 (2,679,703 warp
+# instructions, profiles/outer_residual_128cube_periodic_o4.md); its stencils are 64-bit integer arithmetic.
+RESIDUAL_FP64_PER_CELL = 40.9
 # FP64 peak from unit counts and clocks (the denominator of an ALU-bound kernel): 152 SMs x 2 FP64
 # FMA lanes x 2 flops x 2.07 GHz.  The rate of the library's FMA probe is reported beside it.
 FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.07e9 / 1e12
 # DRAM bytes of one 128^3 residual launch (dram__bytes_read.sum + dram__bytes_write.sum) from one ncu
-# capture (profiles/outer_residual_128cube_periodic_o4.md); None if none
-RESIDUAL_TRAFFIC_128 = None
+# capture (the same file); None if none
+RESIDUAL_TRAFFIC_128 = 161613568 + 57435136
 # the same for the finest colour pass and residual + restriction at 128^3
 # (profiles/smooth_tile_128cube_periodic_o4.md, profiles/restrict_tile_128cube_periodic_o4.md)
 COLOUR_TRAFFIC_128 = 59366656 + 1694976

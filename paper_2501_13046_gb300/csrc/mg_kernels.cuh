@@ -425,14 +425,7 @@ __device__ __forceinline__ void relax_factors(const FaceDiag<T> &fd, const Geo &
     }
 }
 
-// Accessors: value at cell p + (dx, dy, dz) of one field.
-template <typename T>
-struct AccI {   // every offset of the stencil stays inside the box
-    const T *p;
-    int sy, sz;
-    __device__ __forceinline__ T operator()(int dx, int dy, int dz) const { return p[dx + dy * sy + dz * sz]; }
-};
-
+// Accessor: value at cell p + (dx, dy, dz) of one field.
 template <typename T, int BC>
 struct AccB {   // near the boundary; fi: the field (0 = u, 1..3 = W_x..W_z), for symmetry planes
     const T *f;
@@ -491,14 +484,6 @@ __device__ __forceinline__ T dmix(const F &f)
         };
         return (T)(8.0 / 12.0) * (inner(1) - inner(-1)) + (T)(1.0 / 12.0) * (inner(-2) - inner(2));
     }
-}
-
-template <int ORDER>
-__host__ __device__ constexpr int halo() { return ORDER / 2; }
-
-__device__ __forceinline__ bool is_interior(const Geo &g, int i, int j, int k, int G)
-{
-    return i >= G && i < g.n[0] - G && j >= G && j < g.n[1] - G && k >= G && k < g.n[2] - G;
 }
 
 // ---------------------------------------------------------------------------------------

@@ -12,8 +12,8 @@
 // total size 64.  A double within 4 binary orders of E is represented exactly, a smaller one to
 // 2^(E - 57), against the 2^(E - 48) an FP64 sum of the same taps rounds by (16 f + 16 f is
 // formed first).  Only the results are converted: Lap u, the three momentum rows, AtAt.  What is
-// left in FP64 is ~34 instructions per cell (powers of psi, the source terms, the block sums):
-// 128^3 periodic 240 us (integer part alone 165 us, the FP64 part's floor 143 us).
+// left in FP64 is ~40 instructions per cell (powers of psi, the source terms, the block sums):
+// 128^3 periodic 240 us (integer part alone 165 us, the FP64 part's floor ~150 us).
 //
 // March: 16 x 8 cells per plane, one thread per cell, planes along z through a ring of ORDER + 1
 // slots (4 CTAs per SM: their integer and FP64 phases overlap).  The mixed term (1/3) d_i d_j W_j uses
