@@ -80,15 +80,11 @@ inline size_t cluster_smem_bytes(const Geo *lev, int nl, const Geo &gc, int robi
 }
 
 // ---------------------------------------------------------------- cluster primitives
+// All threads of the cluster; orders memory both ways: what was written before it is seen after it, and
+// what was read before it is not overwritten by a write after it (a relaxed arrival orders neither).
 __device__ __forceinline__ void cluster_barrier()
 {
     asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
-}
-
-// The same without ordering of memory: the values read before it have been used, nothing is published.
-__device__ __forceinline__ void cluster_barrier_reads()
-{
-    asm volatile("barrier.cluster.arrive.relaxed;\n\tbarrier.cluster.wait;" ::: "memory");
 }
 
 __device__ __forceinline__ unsigned cluster_rank()
@@ -365,7 +361,8 @@ __global__ void __launch_bounds__(kClusterThreads) k_cluster_cycle(const __grid_
                 nv[it] = row == 0 ? ctr + (fv - Je) / ((ca * dl + cb) * cf.iom)
                                   : ctr + (fv - Je) * (row == 1 ? kW[0] : row == 2 ? kW[1] : kW[2]);
             }
-            if (!(zero && s == 0)) cluster_barrier_reads();   // every CTA has read the old values
+            // every CTA has read the old values (a pass reads cells of its own colour: distance 2, mixed terms)
+            if (!(zero && s == 0)) cluster_barrier();
 #pragma unroll
             for (int it = 0; it < kClusterIts; ++it) {
                 const int lm = sub + it * kStep, m = m0 + lm;
