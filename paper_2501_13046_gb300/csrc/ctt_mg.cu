@@ -644,17 +644,6 @@ mg_status mg_create(const mg_config *cfg, void *cuda_stream, void *workspace, si
                        fused_smem_bytes((int)L1.N, (int)Lc.N, x->tbytes,
                                         fused_ratio_cells(L1.geo, cfg->bc == MG_BC_ROBIN)) <= kMaxCoarseSmem;
         }
-        if (x->dense && x->gamma == 1 && cfg->smoother == 0 && cfg->extrap == 0) {
-            // the first level whose whole bottom fits one cluster's copies (W-cycles and extrapolating faces: as above)
-            const int Lc = x->nlev - 1;
-            for (int l = std::max(0, Lc - kClusterLevels); l < Lc && x->cluster < 0; ++l) {
-                Geo geo[kClusterLevels];
-                for (int k = 0; l + k < Lc; ++k) geo[k] = x->lev[l + k].geo;
-                if (x->lev[l].N <= (size_t)kClusterCells &&
-                    cluster_smem_bytes(geo, Lc - l, x->lev[Lc].geo, cfg->bc == MG_BC_ROBIN, x->tbytes) <= kMaxCoarseSmem)
-                    x->cluster = l;
-            }
-        }
         if (x->dense && (st = ENGINE_CALL(engine_dense_setup, x)) != MG_OK) break;
         if (x->zrhs) {   // the z solve's right-hand side: dF_psi/dK^2 = -psi^5/12 in the psi row's inner form
             cudaError_t e = cudaMemsetAsync(x->zrhs, 0, 4 * x->N * x->tbytes, x->stream);

@@ -79,6 +79,22 @@ inline size_t cluster_smem_bytes(const Geo *lev, int nl, const Geo &gc, int robi
     return s * tb + ints * sizeof(int);
 }
 
+// The level whose bottom the cluster takes: the first one that is small enough, whose copies fit a CTA's shared
+// memory, and of which a cluster with that much per CTA can be placed on this device (placeable(bytes); a
+// partition may have too few free SMs per cluster).  -1: none, the per-level kernels run every level.
+template <class Placeable>
+inline int cluster_level(const Geo *lev, int nlev, int robin, size_t tb, Placeable placeable)
+{
+    const int Lc = nlev - 1;
+    for (int l = Lc > kClusterLevels ? Lc - kClusterLevels : 0; l < Lc; ++l) {
+        const size_t bytes = cluster_smem_bytes(lev + l, Lc - l, lev[Lc], robin, tb);
+        if ((size_t)lev[l].n[0] * lev[l].n[1] * lev[l].n[2] <= (size_t)kClusterCells && bytes <= kMaxCoarseSmem &&
+            placeable(bytes))
+            return l;
+    }
+    return -1;
+}
+
 // ---------------------------------------------------------------- cluster primitives
 // All threads of the cluster; orders memory both ways: what was written before it is seen after it, and
 // what was read before it is not overwritten by a write after it (a relaxed arrival orders neither).

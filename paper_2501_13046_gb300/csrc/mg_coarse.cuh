@@ -17,6 +17,8 @@
 
 namespace ctt {
 
+constexpr size_t kMaxCoarseSmem = 200 * 1024;   // shared memory that a coarse-level CTA may take
+
 constexpr int kDenseMaxW = 400;   // largest bordered W system (3 N + 3) solved densely
 
 __host__ __device__ inline int dense_m_psi(int N, int periodic) { return N + (periodic ? 1 : 0); }

@@ -162,7 +162,6 @@ inline bool dense_eligible(const int nc[3], int periodic)
 }
 
 inline size_t coarse_smem_bytes(size_t Nc, size_t tb) { return 14 * Nc * tb; }
-constexpr size_t kMaxCoarseSmem = 200 * 1024;
 inline size_t direct_smem_bytes(size_t Nc, int periodic, size_t tb)
 {
     size_t m = Nc + (periodic ? 1 : 0);

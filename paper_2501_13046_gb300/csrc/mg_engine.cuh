@@ -173,6 +173,22 @@ mg_status enqueue_coarse(mg_ctx *x, int l)
     return fail(MG_ERR_UNSUPPORTED, "coarsest level too large for the one-CTA coarse solve; use more levels");
 }
 
+// Launch configuration of k_cluster_cycle (attr: storage for its cluster attribute).
+inline cudaLaunchConfig_t cluster_config(size_t smem, cudaStream_t stream, cudaLaunchAttribute *attr)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(kClusterCtas);
+    cfg.blockDim = dim3(kClusterThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    attr->id = cudaLaunchAttributeClusterDimension;
+    attr->val.clusterDim.x = kClusterCtas;
+    attr->val.clusterDim.y = attr->val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cfg;
+}
+
 // The cycle of level l and every level below it in one cluster launch.
 template <typename T, int ORDER, int BC>
 mg_status enqueue_cluster(mg_ctx *x, int l, bool zero)
@@ -203,17 +219,9 @@ mg_status enqueue_cluster(mg_ctx *x, int l, bool zero)
     a.GW = (const T *)x->GW;
     a.mpsi = x->mpsi;
     a.mw = x->mw;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(kClusterCtas);
-    cfg.blockDim = dim3(kClusterThreads);
-    cfg.dynamicSmemBytes = cluster_smem_bytes(geo, a.nl, a.gc, x->cfg.bc == MG_BC_ROBIN, sizeof(T));
-    cfg.stream = x->stream;
     cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeClusterDimension;
-    attr.val.clusterDim.x = kClusterCtas;
-    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
+    const cudaLaunchConfig_t cfg =
+        cluster_config(cluster_smem_bytes(geo, a.nl, a.gc, x->cfg.bc == MG_BC_ROBIN, sizeof(T)), x->stream, &attr);
     CK(cudaLaunchKernelEx(&cfg, k_cluster_cycle<T, ORDER, BC>, a));
     L.curB ^= 1;
     return MG_OK;
@@ -432,7 +440,7 @@ mg_status enqueue_iteration(mg_ctx *x)
 template <typename T, int ORDER, int BC>
 mg_status engine_iteration(mg_ctx *x) { return enqueue_iteration<T, ORDER, BC>(x); }
 
-// Kernel attributes, set once at context creation (never inside a stream capture).
+// Kernel attributes and the choice of the cluster level, once at context creation (never inside a stream capture).
 template <typename T, int ORDER, int BC>
 mg_status engine_prepare(mg_ctx *x)
 {
@@ -463,6 +471,19 @@ mg_status engine_prepare(mg_ctx *x)
                                  (int)kMaxCoarseSmem) != cudaSuccess)
             st = fail(MG_ERR_CUDA, "cudaFuncSetAttribute(k_cluster_cycle)");
     });
+    // the bottom of a V-cycle in one cluster (W-cycles, the untiled reference smoother and extrapolating faces: per level)
+    if (st == MG_OK && x->dense && x->gamma == 1 && x->cfg.smoother == 0 && x->cfg.extrap == 0) {
+        std::vector<Geo> geo;
+        for (const LevelBufs &L : x->lev) geo.push_back(L.geo);
+        x->cluster = cluster_level(geo.data(), x->nlev, x->cfg.bc == MG_BC_ROBIN, sizeof(T), [&](size_t bytes) {
+            cudaLaunchAttribute attr;
+            const cudaLaunchConfig_t cfg = cluster_config(bytes, x->stream, &attr);
+            int n = 0;
+            if (cudaOccupancyMaxActiveClusters(&n, k_cluster_cycle<T, ORDER, BC>, &cfg) == cudaSuccess) return n > 0;
+            (void)cudaGetLastError();   // cannot be placed: no error of the context
+            return false;
+        });
+    }
     return st;
 }
 
