@@ -1474,16 +1474,23 @@ __device__ __forceinline__ void outer_cell(const F &u, const F &w0, const F &w1,
 
 // Pass 2: final residuals, norm partials, inner right-hand side and coefficients in T:
 //   f = (-psi^-5 F_psi, -F_W,i),  a = psi^-5,  b = psi^-5 c,  c = dF_psi/du.
-// F_psi = R0 - (K^2/12) psi^5 and F_W,i = R_i + m_i are always formed in FP64: these are the
-// differences of nearly equal terms.  With an FP32 inner solve (T = float, k_outer_pass2_pairs),
+// F_psi and F_W,i = R_i + m_i are always formed in FP64: these are differences of nearly equal terms.  With an FP32 inner solve (T = float, k_outer_pass2_pairs),
 // the later products (the psi^-5, psi^-6 scalings of H and M, the inner data) are formed in FP32:
 // each is a product of already-accurate factors, so the norms keep 7 significant digits and the
 // FP64 ALU, at 2 lanes per clock per SM on this GPU, is spared the division and powers.
 // Optionally (HM != nullptr) k_outer_pass2 writes H and M (4 FP64 fields, FP64 throughout) instead.
+// F_psi from R0 = Lap u + (1/8) psi^-7 AtAt + 2 pi rho2 psi and its psi^5 terms, which nearly cancel: their factor
+// 2 pi rho0 - K^2/12 is formed first (nk = -K^2/12), so that neither large term is rounded by itself.  (With R0
+// holding 2 pi rho0 psi^5 the norm of |H| at convergence was 1.4e-14 on an 8^3 box, most of it that rounding.)
+__device__ __forceinline__ double f_psi(double R0, double rho0, double p5, double nk)
+{
+    return fma(fma(2.0 * kPi, rho0, nk), p5, R0);
+}
+
 __device__ __forceinline__ float absnanf(float x) { return (x == x) ? fabsf(x) : __int_as_float(0x7f800000); }
 
 // The FP32 inner solve's form, on a colour-split finest level: the two cells of an x pair per thread,
-// 16-byte loads, conversions to FP32 by bits (8 FP64 instructions per cell are left of 17; 5 on boxes
+// 16-byte loads, conversions to FP32 by bits (9 FP64 instructions per cell are left of 18; 6 on boxes
 // without momentum-source means).  128^3: 94 -> 64 us.
 static __global__ void __launch_bounds__(256, 2)
     k_outer_pass2_pairs(Geo g, const double *__restrict__ x, const double *__restrict__ R, const double *__restrict__ src,
@@ -1508,7 +1515,7 @@ static __global__ void __launch_bounds__(256, 2)
             auto of = [&](const double2 &v) { return h == 0 ? v.x : v.y; };
             const double psi = psi_bg(g, (int)i + h, (int)j, (int)k, 2 * pm + h) + of(u2);
             const double p2 = psi * psi, p4 = p2 * p2, p5 = p4 * psi;
-            const double Fp = fma(nk, p5, of(r2));
+            const double Fp = f_psi(of(r2), of(rho02), p5, nk);
             double F0 = of(w02), F1 = of(w12), F2 = of(w22);
             if (shift) {
                 F0 += m[0];
@@ -1564,7 +1571,7 @@ __global__ void __launch_bounds__(256) k_outer_pass2(Geo g, const double *__rest
         const int k = (int)(rest / ny);
         const double psi = psi_bg(g, i, j, k, p) + x[p];
         const double p2 = psi * psi, p4 = p2 * p2, p5 = p4 * psi;
-        const double Fp = fma(nk, p5, R[p]);
+        const double Fp = f_psi(R[p], src[p], p5, nk);
         const double Fw0 = R[N + p] + m0, Fw1 = R[2 * N + p] + m1, Fw2 = R[3 * N + p] + m2;
         const double ip = recip_f64(psi), ip2 = ip * ip, ip5 = ip2 * ip2 * ip, ip6 = ip5 * ip;
         const double H = -8.0 * ip5 * Fp;

@@ -46,7 +46,8 @@ mg_status scratch_address(double **out)
 
 // Maxima of |H| and |M_i|, finished in the last block.
 __global__ void __launch_bounds__(256) k_noalloc_norms(Geo g, const double *__restrict__ u,
-                                                       const double *__restrict__ R, Scalars *s,
+                                                       const double *__restrict__ R,
+                                                       const double *__restrict__ rho0, Scalars *s,
                                                        double *__restrict__ partial)
 {
     const size_t N = (size_t)g.n[0] * g.n[1] * g.n[2];
@@ -60,7 +61,7 @@ __global__ void __launch_bounds__(256) k_noalloc_norms(Geo g, const double *__re
         double psi = psi_background(g, i, j, k) + u[p];
         double p2 = psi * psi, p4 = p2 * p2, p5 = p4 * psi;
         double ip = recip_f64(psi), ip2 = ip * ip, ip5 = ip2 * ip2 * ip, ip6 = ip5 * ip;
-        max_abs(mxu[0], -8.0 * ip5 * fma(nk, p5, R[p]));
+        max_abs(mxu[0], -8.0 * ip5 * f_psi(R[p], rho0[p], p5, nk));
 #pragma unroll
         for (int a = 0; a < 3; ++a) max_abs(mxu[1 + a], ip6 * (R[(1 + a) * N + p] + m[a]));
     }
@@ -160,7 +161,7 @@ extern "C" mg_status mg_residual_norms_noalloc(const mg_config *cfg, const doubl
         if (cfg->bc == MG_BC_PERIODIC) launch1(I4(), P()); else launch1(I4(), Rb());
     }
     CK(attr);
-    k_noalloc_norms<<<g1, kThreads, 0, st>>>(g, u, R, sc, partial);
+    k_noalloc_norms<<<g1, kThreads, 0, st>>>(g, u, R, rho0, sc, partial);
     CK(cudaGetLastError());
     Scalars h;
     CK(cudaMemcpyAsync(&h, sc, sizeof(Scalars), cudaMemcpyDeviceToHost, st));
