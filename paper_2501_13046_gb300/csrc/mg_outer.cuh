@@ -97,8 +97,10 @@ inline OuterInt make_outer_int(const Geo &g, int order)
 {
     OuterInt o;
     const double hmin = fmin(g.h[0], fmin(g.h[1], g.h[2])), hmax = fmax(g.h[0], fmax(g.h[1], g.h[2]));
-    o.iso = hmax <= hmin * (1.0 + 4.5e-16);   // the same spacing up to the rounding of (hi - lo) / n
-    const long double hb = hmin;
+    // equal spacings, or one unit of the last place apart as (hi - lo) / n may leave them: their mean is then as near to
+    // each as a rounded 1/h^2 is to its own
+    o.iso = hmax <= nextafter(hmin, hmax);
+    const long double hb = o.iso ? ((long double)hmin + (long double)hmax) / 2 : (long double)hmin;
     auto fix = [](long double v, int bits) {  // v 2^bits, at most 2^63 - 1
         const long double s = ldexpl(v, bits);
         return s >= 9223372036854775807.0L ? 9223372036854775807LL : (long long)(s + 0.5L);
@@ -641,17 +643,17 @@ __global__ void __launch_bounds__(kOutThreads, 4)
                 for (int A = 0; A < 3; ++A) {
                     long long any = 0;
 #pragma unroll
-                    for (int a = 0; a < 3; ++a) {
-                        if (!oi.iso) g9[a][A] = __mul64hi(g9[a][A] << 1, oi.ga[a]);
-                        any |= g9[a][A] ^ (g9[a][A] >> 63);
-                    }
+                    for (int a = 0; a < 3; ++a) any |= g9[a][A] ^ (g9[a][A] >> 63);
                     if (any) U = max(U, Ew[A] + 3 - __clzll(any));
                 }
 #pragma unroll
                 for (int A = 0; A < 3; ++A) {
                     const int n = Ew[A] - U, l = min(63, max(n, 0)), r = min(63, max(-n, 0));
 #pragma unroll
-                    for (int a = 0; a < 3; ++a) g9[a][A] = g9[a][A] << l >> r;
+                    for (int a = 0; a < 3; ++a) {
+                        g9[a][A] = g9[a][A] << l >> r;
+                        if (!oi.iso) g9[a][A] = __mul64hi(g9[a][A] << 1, oi.ga[a]);   // (after the shift: no bits are lost)
+                    }
                 }
                 constexpr long long kThird = 0x5555555555555555LL;   // 2^64 / 3
                 const long long third = __mul64hi(g9[0][0] + g9[1][1] + g9[2][2], kThird);
