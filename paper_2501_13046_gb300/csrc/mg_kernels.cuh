@@ -1297,18 +1297,19 @@ __global__ void __launch_bounds__(256) k_sum4(const T *__restrict__ x, size_t N,
 #pragma unroll
                 for (int a = 0; a < 4; ++a) two_sum_add(hi[a][0], lo[a][0], (float)x[a * N + p]);
         }
-        // the pairs of a warp are added as pairs too: one FP64 conversion per warp, not per thread
+        // every sum beyond the thread in FP64 (a float pair holds 48 bits).  Lanes exchange fields while they add, so that
+        // a warp's four sums take 6 additions a lane, not 20: lane 8 a ends with field a
 #pragma unroll
-        for (int a = 0; a < 4; ++a) {
-            two_sum_add(hi[a][0], lo[a][0], hi[a][1]);
-            lo[a][0] += lo[a][1];
-            for (int o = 16; o > 0; o >>= 1) {
-                const float h = __shfl_xor_sync(0xffffffffu, hi[a][0], o), l = __shfl_xor_sync(0xffffffffu, lo[a][0], o);
-                two_sum_add(hi[a][0], lo[a][0], h);
-                lo[a][0] += l;
-            }
-            if ((threadIdx.x & 31) == 0) sw[threadIdx.x >> 5][a] = (double)hi[a][0] + (double)lo[a][0];
-        }
+        for (int a = 0; a < 4; ++a) v[a] = (to_f64(hi[a][0]) + to_f64(lo[a][0])) + (to_f64(hi[a][1]) + to_f64(lo[a][1]));
+        const int lane = threadIdx.x & 31;
+        const bool up = lane & 16, second = lane & 8;
+        double w0 = up ? v[2] : v[0], w1 = up ? v[3] : v[1];
+        w0 += __shfl_xor_sync(0xffffffffu, up ? v[0] : v[2], 16);
+        w1 += __shfl_xor_sync(0xffffffffu, up ? v[1] : v[3], 16);
+        double w = (second ? w1 : w0) + __shfl_xor_sync(0xffffffffu, second ? w0 : w1, 8);
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
+        if ((lane & 7) == 0) sw[threadIdx.x >> 5][lane >> 3] = w;
         __syncthreads();
         if (threadIdx.x < 4) {
             double t = 0.0;
