@@ -60,10 +60,10 @@ __global__ void __launch_bounds__(256) k_noalloc_norms(Geo g, const double *__re
         int k = (int)(rest / g.n[1]);
         double psi = psi_background(g, i, j, k) + u[p];
         double p2 = psi * psi, p4 = p2 * p2, p5 = p4 * psi;
-        double ip = recip_f64(psi), ip2 = ip * ip, ip5 = ip2 * ip2 * ip, ip6 = ip5 * ip;
-        max_abs(mxu[0], -8.0 * ip5 * f_psi(R[p], rho0[p], p5, nk));
+        const PsiInverse inv = psi_inverse(psi, p5);
+        max_abs(mxu[0], -8.0 * inv.i5 * f_psi(R[p], rho0[p], p5, nk));
 #pragma unroll
-        for (int a = 0; a < 3; ++a) max_abs(mxu[1 + a], ip6 * (R[(1 + a) * N + p] + m[a]));
+        for (int a = 0; a < 3; ++a) max_abs(mxu[1 + a], inv.i6 * (R[(1 + a) * N + p] + m[a]));
     }
     double mx[4], r[4];
 #pragma unroll
