@@ -614,16 +614,15 @@ SplitPlan split_plan(long long nvox)
 template <int CIN, int COUT>
 int launch_fwd(const ConvArgs &a, int nvox, float *ws, cudaStream_t st)
 {
-    // block-tile kernel where the grid tiles evenly and the block and all weights fit in shared
-    // memory: it reads each input voxel about 3 times (halo), the per-tap kernel 27 times (L2)
+    // Block-tile kernel where the grid tiles evenly and the block and all weights fit in shared
+    // memory: it reads each input voxel about 3 times (halo), the per-tap kernel 27 times (L2).  Measured from 8 to
+    // 1024 tiles (16 x 16 x 8 to 64^3 voxels), block tile against taps, us: 16 -> 16 channels 6.4 and 14.5 against 14.5 and
+    // 48; 32 -> 64 12.5 and 74 against 17.6 and 137; 32 -> 96 18.6 and 115 against 22.7 and 173; 64 -> 32 18.6 and 119 against 16.5
+    // and 316 (its 8 tiles are the one size where the taps are ahead; at 32 tiles 18.6 against 22.7): no rule on the size.
     constexpr int ZT = 2;
     constexpr size_t bsm = blk_smem_bytes<CIN, COUT, ZT>();
     if constexpr (bsm <= 220 * 1024) {
-        // the largest layers (64 -> 32, 32 -> 96: block and weights near the limit) only on grids of at
-        // least 96 blocks: below, the split taps spread the work over more SMs
-        constexpr bool large = (CIN == 64 && COUT == 32) || (CIN == 32 && COUT == 96);
-        const long long tiles = (long long)(a.n0 / kBlkX) * (a.n1 / kBlkY) * (a.n2 / ZT);
-        if (a.n0 % kBlkX == 0 && a.n1 % kBlkY == 0 && a.n2 % ZT == 0 && (!large || tiles >= 96)) {
+        if (a.n0 % kBlkX == 0 && a.n1 % kBlkY == 0 && a.n2 % ZT == 0) {
             static bool attr_blk = false;
             if (!attr_blk) {
                 if (cudaFuncSetAttribute(k_conv3d_blk<CIN, COUT, ZT>, cudaFuncAttributeMaxDynamicSharedMemorySize,

@@ -12,7 +12,7 @@ from tests.test_gpu_unet_conv import U, bf16, tohost  # noqa: E402,F401
 
 
 @pytest.mark.parametrize("cin,cout", [(64, 32), (32, 96), (32, 64)])
-@pytest.mark.parametrize("shape", [(32, 32, 24), (16, 48, 40)])   # 96 and 120 tiles of 8 x 16 x 2 voxels
+@pytest.mark.parametrize("shape", [(8, 16, 2), (16, 16, 8), (32, 32, 24), (16, 48, 40)])   # 1, 8, 96, 120 tiles of 8 x 16 x 2
 def test_conv_forward_block_tiles_of_large_layers(U, cin, cout, shape):  # noqa: F811
     nx, ny, nz = shape
     rng = np.random.default_rng(cin * 977 + cout + nx)
