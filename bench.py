@@ -291,15 +291,16 @@ def batch_measure(mg, torch, sp, precision, repeats=1):
             "max_norm": max(float(i["norms"].max()) for i in infos)}
 
 
-# FP64-pipe instructions of the fused residual per cell, from one ncu capture at 128^3 (2,679,703 warp
-# instructions, profiles/outer_residual_128cube_periodic_o4.md); its stencils are 64-bit integer arithmetic.
-RESIDUAL_FP64_PER_CELL = 40.9
-# FP64 peak from unit counts and clocks (the denominator of an ALU-bound kernel): 152 SMs x 2 FP64
-# FMA lanes x 2 flops x 2.07 GHz.  The rate of the library's FMA probe is reported beside it.
-FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.07e9 / 1e12
+# FP64-pipe instructions of the fused residual per cell (multiply-adds, additions, conversions), from one ncu capture
+# at 128^3 (3,332,789 warp instructions, profiles/outer_residual_128cube_periodic_o4.md); its stencils are 64-bit integer
+# arithmetic.
+RESIDUAL_FP64_PER_CELL = 50.9
+# Issue slots of the FP64 pipe per second from unit counts and clocks (the denominator of an ALU-bound kernel): 152 SMs x 2
+# lanes x 2.07 GHz.  A slot holds any FP64 instruction, so this is the pipe's occupancy and no rate of flops.
+FP64_PEAK_TSLOTS = 152 * 2 * 2.07e9 / 1e12
 # DRAM bytes of one 128^3 residual launch (dram__bytes_read.sum + dram__bytes_write.sum) from one ncu
 # capture (the same file); None if none
-RESIDUAL_TRAFFIC_128 = 161613568 + 57435136
+RESIDUAL_TRAFFIC_128 = 161633536 + 56829952
 # the same for the finest colour pass and residual + restriction at 128^3
 # (profiles/smooth_tile_128cube_periodic_o4.md, profiles/restrict_tile_128cube_periodic_o4.md)
 COLOUR_TRAFFIC_128 = 59366656 + 1694976
@@ -313,15 +314,15 @@ def kernel_rooflines(mg, ctx, N):
     ms0, bytes0 = mg.mg_time_kernel(ctx, 0, 40)   # finest FP32 colour pass
     ms1, bytes1 = mg.mg_time_kernel(ctx, 1, 20)   # finest residual + restriction
     fp64 = mg.mg_fp64_fma_rate(ctx, 3)           # FP64 FMA rate of the library probe (context)
-    ach = 2 * RESIDUAL_FP64_PER_CELL * N / (msb * 1e-3) / 1e12   # an issue slot counts as one FMA
+    ach = RESIDUAL_FP64_PER_CELL * N / (msb * 1e-3) / 1e12
     sm_gbs = bytes0 / (ms0 * 1e-3) / 1e9
     rr_gbs = bytes1 / (ms1 * 1e-3) / 1e9
-    return {"bound": "alu", "achieved": ach, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
-            "frac": ach / FP64_PEAK_TFLOPS, "traffic": RESIDUAL_TRAFFIC_128 if N == 128 ** 3 else None,
+    return {"bound": "alu", "achieved": ach, "peak": FP64_PEAK_TSLOTS, "unit": "1e12 FP64 issue slots/s",
+            "frac": ach / FP64_PEAK_TSLOTS, "traffic": RESIDUAL_TRAFFIC_128 if N == 128 ** 3 else None,
             "kernel": "k_outer_residual<4,periodic> (fused FP64 residual, 128^3; FP64 and integer pipes)",
             "ms_per_launch": msb, "fp64_issue_slots": RESIDUAL_FP64_PER_CELL * N, "algorithmic_bytes": bytesb,
-            "peak_source": "derived: 152 SMs x 2 FP64 FMA lanes x 2 flops x 2.07 GHz",
-            "fp64_probe_tflops": fp64, "frac_of_probe": ach / fp64,
+            "peak_source": "derived: 152 SMs x 2 FP64 lanes x 2.07 GHz",
+            "fp64_probe_tflops": fp64, "frac_of_probe": 2 * ach / fp64,
             "colour_pass": {"bound": "hbm", "kernel": "k_smooth_tile<float,4,periodic,c> (finest, one colour)",
                             "ms_per_launch": ms0, "algorithmic_bytes": bytes0, "achieved": sm_gbs,
                             "unit": "GB/s", "peak": pk["hbm_gbs"], "frac": sm_gbs / pk["hbm_gbs"],

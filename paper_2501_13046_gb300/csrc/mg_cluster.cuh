@@ -8,8 +8,10 @@
 // every level in its shared memory; a step's cells are split over the CTAs, and a new value is
 // written to all 8 copies through distributed shared memory, so neighbours are always local reads
 // and no halo exists.  One step costs its longest thread's stencil (4400 cycles at 16^3, 1900 at 8^3), its
-// stores (~1500) and one or two cluster barriers (~300 and ~1200): 47 us per V(1,1) cycle from 16^3 down in
-// 4th order, where the per-level kernels took 78.  FP64 from 8^3 down: 39 us against 175 us in one CTA.
+// stores (~1500) and one or two cluster barriers: 42 us per V(1,1) cycle from 16^3 down in 4th order back to back
+// (Robin 76; 56 and 96 cold, between other kernels), where the per-level kernels took 78.  FP64 from 8^3 down: 29 us
+// against 175 us in one CTA.  The cluster barriers are hardware barriers of one launch, whose 8 CTAs run together by
+// definition and all reach every one of them: no wait on a flag, so no iteration limit.
 //
 // A warp takes one row of the operator (psi, W_x, W_y or W_z) at 32 cells, so a thread's chain is
 // one row's taps (13 or 45 in 4th order), not all four rows' 148.  Shared-memory layout of a field:

@@ -1267,7 +1267,7 @@ static __global__ void __launch_bounds__(256) k_flag_nonfinite(const double *__r
 
 // Sums of 4 contiguous fields (block partials); with means != nullptr the last block also forms
 // means[a] = sum_a / N (ticket: its finalize_last counter).  Fields of a multiple of 4 cells (every
-// grid with more than one level) are read 16 bytes at a time.  128^3 FP32: 35 -> 18 us.
+// grid with more than one level) are read 16 bytes at a time.  128^3 FP32: 35 -> 19 us.
 constexpr int kSumBlocks = 152 * 2;
 
 // s + b as an unevaluated pair hi + lo of floats, exact (Knuth's two-sum; the rounding error of every addition
@@ -1503,7 +1503,7 @@ __device__ __forceinline__ float absnanf(float x) { return (x == x) ? fabsf(x) :
 
 // The FP32 inner solve's form, on a colour-split finest level: the two cells of an x pair per thread,
 // 16-byte loads, conversions to FP32 by bits (9 FP64 instructions per cell are left of 18; 6 on boxes
-// without momentum-source means).  128^3: 94 -> 64 us.
+// without momentum-source means).  128^3: 94 -> 67 us.
 static __global__ void __launch_bounds__(256, 2)
     k_outer_pass2_pairs(Geo g, const double *__restrict__ x, const double *__restrict__ R, const double *__restrict__ src,
                         Scalars *s, float *__restrict__ f, float *__restrict__ ab, double *__restrict__ partial)
