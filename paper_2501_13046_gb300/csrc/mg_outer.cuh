@@ -17,7 +17,7 @@
 // packed into full warps; that is one cell in thousands of smooth fields (a field and its gradient small together),
 // and all cells outside a steep peak.  Where the values of a whole window have fallen kOutFall
 // binary orders below E, the march starts anew in smaller units (it costs about three planes).  Zeros stay exact.
-// Against 128-bit arithmetic: see tests/test_gpu_outer_local.py.
+// Every cell is held to a bound from its own taps by tests/test_gpu_outer_local.py, which also prints the errors.
 //
 // What is left in FP64 is 51 instructions per cell (powers of psi, the source terms, the sums of different fields,
 // the block sums), 170 us of that pipe at 128^3 periodic; the kernel takes 312 us there (the two FP64 kernels 684), 2016

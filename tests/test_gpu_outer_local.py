@@ -45,8 +45,8 @@ def along(a, s):
     return tuple(s if c == a else 0 for c in range(3))
 
 
-def reference(order, h, u, W):
-    """H, M of a vacuum state with K = 0 on a periodic box, and their bounds."""
+def reference(order, h, u, W, src=None, K=0.0):
+    """H, M of a state on a periodic box (src: rho0, rho2, S; None: vacuum), and their bounds."""
     F1 = {1: L(1) / 2, -1: -L(1) / 2} if order == 2 else {1: L(8) / 12, -1: -L(8) / 12, 2: -L(1) / 12, -2: L(1) / 12}
     F2 = ({0: L(-2), 1: L(1), -1: L(1)} if order == 2 else
           {0: -L(30) / 12, 1: L(16) / 12, -1: L(16) / 12, 2: -L(1) / 12, -2: -L(1) / 12})
@@ -81,20 +81,31 @@ def reference(order, h, u, W):
             aa, aa_err = aa + at * at, aa_err + 2 * np.abs(at) * de + de * de
     psi = 1 + u
     nl = aa / (8 * psi ** 7)
-    H = -8 * (lap + nl) / psi ** 5
-    tol_H = 8 / psi ** 5 * (lap_err + aa_err / (8 * psi ** 7) + 32 * EPS * (np.abs(lap) + nl))
-    M = np.stack(mom) / psi ** 6
-    tol_M = (np.stack(mom_err) + 32 * EPS * np.abs(np.stack(mom))) / psi ** 6
-    return H, M, tol_H, tol_M
+    F, terms = lap + nl, np.abs(lap) + nl
+    mom, mom_err = np.stack(mom), np.stack(mom_err) + 32 * EPS * np.abs(np.stack(mom))
+    if src is not None:
+        pi = L("3.14159265358979323846264338327950288")
+        rho0, rho2, S = (f.astype(L) for f in src)
+        F = F + 2 * pi * (rho0 * psi ** 5 + rho2 * psi) - L(K) ** 2 / 12 * psi ** 5
+        terms = terms + 2 * pi * (np.abs(rho0) * psi ** 5 + np.abs(rho2) * psi) + L(K) ** 2 / 12 * psi ** 5
+        s = 8 * pi * psi ** 6 * S
+        mean = s.mean(axis=(1, 2, 3), keepdims=True)
+        mom = mom - s + mean
+        # (a mean's sum rounds once per term at most)
+        mom_err = mom_err + 32 * EPS * np.abs(s) + (s[0].size ** 0.5 + 64) * EPS * np.abs(s).mean(axis=(1, 2, 3), keepdims=True)
+    H = -8 * F / psi ** 5
+    tol_H = 8 / psi ** 5 * (lap_err + aa_err / (8 * psi ** 7) + 32 * EPS * terms)
+    return H, mom / psi ** 6, tol_H, mom_err / psi ** 6
 
 
-def gpu_fields(mg, n, h, order, u, W):
+def gpu_fields(mg, n, h, order, u, W, src=None, K=0.0):
     p = dict(n=list(n), lo=[0.0] * 3, hi=[h[a] * n[a] for a in range(3)], order=order, bc=fields.PERIODIC,
-             kmode=fields.K_FIXED, K=0.0, punctures=[])
+             kmode=fields.K_FIXED, K=K, punctures=[])
     z = np.zeros_like(u)
+    rho0, rho2, S = src if src is not None else (z, z, [z] * 3)
     ctx = mg.mg_create(mg.config_for(p, mg.MG_FP64), torch.cuda.current_stream().cuda_stream)
     try:
-        mg.mg_set_sources(ctx, z, z, z, z, z)
+        mg.mg_set_sources(ctx, *[np.ascontiguousarray(f) for f in (rho0, rho2, *S)])
         mg.mg_set_initial_guess(ctx, np.ascontiguousarray(u), np.ascontiguousarray(W))
         H, M = np.empty_like(u), np.empty_like(W)
         mg.mg_constraint_fields(ctx, H, M)
@@ -103,9 +114,11 @@ def gpu_fields(mg, n, h, order, u, W):
     return H, M
 
 
-def check(mg, n, h, order, u, W):
-    H, M = gpu_fields(mg, n, h, order, u, W)
-    rH, rM, tol_H, tol_M = reference(order, h, u, W)
+def check(mg, n, h, order, u, W, src=None, K=0.0):
+    H, M = gpu_fields(mg, n, h, order, u, W, src, K)
+    rH, rM, tol_H, tol_M = reference(order, h, u, W, src, K)
+    l2 = lambda a, b: float(np.sqrt(((a - b) ** 2).sum() / np.maximum((b ** 2).sum(), L(1e-300))))
+    print("order %d, spacings %s: relative L2 error of H %.2e, of M %.2e" % (order, h, l2(H, rH), l2(M, rM)))
     tiny = 1e-290   # (squares and products below the smallest normal number)
     assert (np.abs(H - rH) <= tol_H + tiny).all(), float(np.max(np.abs(H - rH) / (tol_H + tiny)))
     for a in range(3):
@@ -169,3 +182,21 @@ def test_zeros_stay_zero(mg):
         near = np.zeros(u.shape, bool)
         near[8:16, 2:10, 1:8] = True
         assert (H[~near] == 0).all() and (M[:, ~near] == 0).all()
+
+
+@pytest.mark.parametrize("h", SPACINGS)
+@pytest.mark.parametrize("order", [2, 4])
+def test_smooth_state_with_matter(mg, order, h):
+    """A state on its way to the solution: smooth u and W, a nearly uniform scalar field's sources and the K of their mean."""
+    rng = np.random.default_rng(2)
+    x = [np.arange(N[a]).reshape([-1 if b == 2 - a else 1 for b in range(3)]) / N[a] for a in range(3)]
+
+    def modes(amplitude):
+        f = np.zeros(N[::-1])
+        for _ in range(8):
+            k = rng.integers(-3, 4, 3)
+            f += amplitude / (1 + np.abs(k).sum()) * np.cos(2 * np.pi * sum(k[a] * x[a] for a in range(3)) + 2 * np.pi * rng.random())
+        return f
+    u, W = modes(0.01), np.stack([modes(1e-3) for _ in range(3)])
+    rho0, rho2, S = 0.5 + modes(1e-3), modes(1e-4) ** 2, np.stack([modes(1e-5) for _ in range(3)])
+    check(mg, N, h, order, u, W, (rho0, rho2, S), K=-np.sqrt(24 * np.pi * rho0.mean()))
